@@ -121,7 +121,7 @@ svv_status svv_build_versioned_csr(uint32_t V, uint32_t S, uint64_t n_inst, cons
  * copies them and the caller keeps ownership.  Internally each row is reordered
  * so that edges present in all S snapshots come first (Section 4.1), and edges
  * present in no snapshot are dropped.  Unless the "pull" tuning key is 0, a
- * transposed copy (in-edges sorted by target, 12 bytes per edge plus the masks
+ * transposed copy (in-edges grouped by target, 8 bytes per edge plus the masks
  * of partial edges) is kept as well for the solves' pull rounds.  Replaces any
  * graph loaded before.
  * SVV_EINVAL on a malformed CSR, S == 0, V >= 2^32-1 or E >= 2^32;
@@ -399,7 +399,7 @@ svv_status svv_autotune(svv_ctx *ctx, svv_type type, uint32_t source, uint32_t w
  * with device outputs whose windows have one length of at most 128 snapshots
  * relaxes both queries in one launch over both queries' rows; 0 relaxes them
  * one after the other; results identical), "group_pull_pct" /
- * "group_pull_pct_union" (0..100, defaults 15 / 100: a group's intersection /
+ * "group_pull_pct_union" (0..100, defaults 5 / 10: a group's intersection /
  * union solve pulls when its frontier holds more than this % of all work
  * units; 0 or 100 = push only), "isolated_fast" (1 default: a query whose
  * source has no out-edge in any snapshot is answered by one fill -- the

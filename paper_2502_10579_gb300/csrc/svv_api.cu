@@ -127,7 +127,7 @@ SolveArgs solve_base(svv_ctx* c, uint32_t wb, uint32_t wl, int type, const Knobs
   const uint64_t cap = a.delta ? 16ull * c->g.V + 64 : (uint64_t)c->g.V + 2;
   a.maxit = c->maxit ? c->maxit : (uint32_t)std::min<uint64_t>(cap, 0xFFFFFFF0ull);
   a.spin_ns = (unsigned long long)c->spin_ms * 1000000ull;
-  if (c->g.ifd && kn.pull_pct) {
+  if (c->g.pull && kn.pull_pct) {
     const uint64_t all_units = (uint64_t)c->g.V + (c->g.E >> kn.solve_cs);
     a.pull_units = (uint32_t)std::max<uint64_t>(1, all_units * kn.pull_pct / 100);
     a.push_verts = (uint32_t)std::max<uint64_t>(1, (uint64_t)c->g.V * kn.pull_pct / 100);
@@ -443,46 +443,6 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
     }
   }
 
-  // transposed graph, edge-flat: in-edges sorted by target (counting sort;
-  // sources ascending within a target), all-snapshot ones and partial ones
-  // (with their masks) in separate arrays
-  const uint32_t EF = E2 - NF;
-  std::vector<uint32_t> ifd, ipd;
-  std::vector<uint2> ifcw, ipcw;
-  std::vector<uint64_t> ipm;
-  if (c->pull) {
-    std::vector<uint32_t> pos_f((size_t)V + 1, 0), pos_p((size_t)V + 1, 0);
-    for (uint32_t u = 0; u < V; ++u) {
-      const uint32_t fe = rp[u + 1] - (nfp[u + 1] - nfp[u]);
-      for (uint32_t e = rp[u]; e < rp[u + 1]; ++e) (e < fe ? pos_f : pos_p)[cw[e].x + 1]++;
-    }
-    for (uint32_t v = 0; v < V; ++v) {
-      pos_f[v + 1] += pos_f[v];
-      pos_p[v + 1] += pos_p[v];
-    }
-    ifd.assign(std::max<uint32_t>(EF, 1), 0u);
-    ifcw.assign(std::max<uint32_t>(EF, 1), make_uint2(0, 0));
-    ipd.assign(std::max<uint32_t>(NF, 1), 0u);
-    ipcw.assign(std::max<uint32_t>(NF, 1), make_uint2(0, 0));
-    ipm.assign((size_t)std::max<uint32_t>(NF, 1) * W, 0ull);
-    for (uint32_t u = 0; u < V; ++u) {
-      const uint32_t fe = rp[u + 1] - (nfp[u + 1] - nfp[u]);
-      for (uint32_t e = rp[u]; e < rp[u + 1]; ++e) {
-        const uint32_t x = cw[e].x;
-        if (e < fe) {
-          const uint32_t i2 = pos_f[x]++;
-          ifd[i2] = x;
-          ifcw[i2] = make_uint2(u, cw[e].y);
-        } else {
-          const uint32_t k = pos_p[x]++;
-          ipd[k] = x;
-          ipcw[k] = make_uint2(u, cw[e].y);
-          for (uint32_t w = 0; w < W; ++w) ipm[(size_t)k * W + w] = nfm[(size_t)(nfp[u] + (e - fe)) * W + w];
-        }
-      }
-    }
-  }
-
   // replace the resident graph
   cudaDeviceSynchronize();
   free_graph(c);
@@ -528,34 +488,6 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
   g.nfmask = d_nfm;
   g.nfsrc = d_nfsrc;
   g.nfcw = d_nfcw;
-  if (c->pull) {
-    uint32_t *d_ifd, *d_ipd;
-    uint2 *d_ifcw, *d_ipcw;
-    uint64_t* d_ipm;
-    if ((st = alloc_n(c, c->graph_bufs, std::max<uint32_t>(EF, 1), &d_ifd)) ||
-        (st = alloc_n(c, c->graph_bufs, std::max<uint32_t>(EF, 1), &d_ifcw)) ||
-        (st = alloc_n(c, c->graph_bufs, std::max<uint32_t>(NF, 1), &d_ipd)) ||
-        (st = alloc_n(c, c->graph_bufs, std::max<uint32_t>(NF, 1), &d_ipcw)) ||
-        (st = alloc_n(c, c->graph_bufs, (uint64_t)std::max<uint32_t>(NF, 1) * W, &d_ipm))) {
-      free_graph(c);
-      return st;
-    }
-    cudaError_t e2 = cudaMemcpy(d_ifd, ifd.data(), (size_t)EF * 4, cudaMemcpyHostToDevice);
-    if (e2 == cudaSuccess) e2 = cudaMemcpy(d_ifcw, ifcw.data(), (size_t)EF * 8, cudaMemcpyHostToDevice);
-    if (e2 == cudaSuccess) e2 = cudaMemcpy(d_ipd, ipd.data(), (size_t)NF * 4, cudaMemcpyHostToDevice);
-    if (e2 == cudaSuccess) e2 = cudaMemcpy(d_ipcw, ipcw.data(), (size_t)NF * 8, cudaMemcpyHostToDevice);
-    if (e2 == cudaSuccess) e2 = cudaMemcpy(d_ipm, ipm.data(), (size_t)NF * W * 8, cudaMemcpyHostToDevice);
-    if (e2 != cudaSuccess) {
-      free_graph(c);
-      return cuda_fail(c, e2, "uploading the transposed graph");
-    }
-    g.ifd = d_ifd;
-    g.ifcw = d_ifcw;
-    g.ipd = d_ipd;
-    g.ipcw = d_ipcw;
-    g.ipmask = d_ipm;
-  }
-
   // scratch sized from V and E
   const uint64_t qcap = (uint64_t)V + E2 / (1u << std::min(c->solve_cs, c->relax_cs)) + 64;
   const uint64_t ucap = (uint64_t)V + E2 / (1u << c->qrs_cs) + 64;
@@ -582,6 +514,10 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
   c->pcap = (uint32_t)((uint64_t)V + (E2 >> 4) + 64);
   c->ecap = std::max<uint32_t>(E2, 1);
   c->g = g;
+  if (c->pull && (st = build_pull(c))) {
+    free_graph(c);
+    return st;
+  }
   // out-degree over the edges present in some snapshot: a source without any
   // reaches nothing in any window (the query's result is known without a solve)
   c->hdeg.resize(V);

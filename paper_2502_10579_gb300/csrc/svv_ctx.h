@@ -153,7 +153,11 @@ struct svv_ctx {
   bool skip_same = true;                // per-chunk last-relaxed value (procv)
   uint32_t relax_lanes = 32;            // lanes per edge in the relaxation (8, 16, 32)
   bool pull = true;                     // build the transposed graph at load; pull dense rounds
-  uint32_t pull_pct = 15;               // pull when the frontier holds > pull_pct % of all units
+  // Pull when the frontier holds > pull_pct % of all units.  A pull round costs
+  // about the same whatever the frontier (20-45 us at 1M vertices, 16.8M
+  // edges); a push round from 5% of the units costs 45 us, from 8% 57 us.
+  // 15 -> 5: the scale-20 solves 1-10% faster, 8 / 3 / 2 within 2% of 5.
+  uint32_t pull_pct = 5;
   uint32_t* procv = nullptr;
   uint32_t pcap = 0;
   cudaEvent_t ev[7] = {};
@@ -229,9 +233,10 @@ struct svv_ctx {
   // query groups: lane rows of the two bounds, per-lane planar copies, lane
   // words of the partial edges, the group's error word
   uint32_t group_max = svv::kGroupMax;  // queries per group (1 = every query alone)
-  // pull threshold of the group solves (intersection, union), % of all units:
-  // a group pull round gathers a whole lane row per in-edge, so groups pull later
-  uint32_t group_pull_pct[2] = {15, 100};
+  // pull threshold of the group solves (intersection, union), % of all units
+  // (scale-22 batch of 16: 11.32 ms at 15 / 100, 11.24 at 5 / 100, 10.93 at
+  // 5 / 5, 10.95 at 5 / 10; the union's frontier is small and rarely passes 10%)
+  uint32_t group_pull_pct[2] = {5, 10};
   bool group_mix = false;  // groups may hold queries of different types
   int occ_group = 0;   // group solves of 4 or 8 lanes
   int occ_group2 = 0;  // of 2 lanes
@@ -329,6 +334,8 @@ inline void slab_shape(uint32_t ls, uint32_t& P, uint32_t& K) {
     K = 4;
   }
 }
+
+svv_status build_pull(svv_ctx* c);  // the transposed graph (svv_layout.cu)
 
 // host helpers of the query pipeline (svv_api.cu)
 struct CompactOut {

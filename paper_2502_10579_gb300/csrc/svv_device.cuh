@@ -226,7 +226,7 @@ struct OpSSSP {  // CASMIN(Val(v), Val(u) + w), saturating
     unsigned long long s = (unsigned long long)sv + w;
     return s > kSat ? kSat : (uint32_t)s;
   }
-  __device__ __forceinline__ static bool better(uint32_t a, uint32_t b) { return a < b; }
+  __host__ __device__ __forceinline__ static constexpr bool better(uint32_t a, uint32_t b) { return a < b; }
   __device__ __forceinline__ static uint32_t atomic(uint32_t* p, uint32_t v) { return atomicMin(p, v); }
   __device__ __forceinline__ static void red(uint32_t* p, uint32_t v) { atomicMin(p, v); }  // no return: a reduction
 };
@@ -236,7 +236,7 @@ struct OpSSWP {  // CASMAX(Val(v), min(Val(u), w))
   static constexpr uint32_t kIdentity = 0;
   static constexpr uint32_t kSource = kInf;
   __device__ __forceinline__ static uint32_t relax(uint32_t sv, uint32_t w) { return sv < w ? sv : w; }
-  __device__ __forceinline__ static bool better(uint32_t a, uint32_t b) { return a > b; }
+  __host__ __device__ __forceinline__ static constexpr bool better(uint32_t a, uint32_t b) { return a > b; }
   __device__ __forceinline__ static uint32_t atomic(uint32_t* p, uint32_t v) { return atomicMax(p, v); }
   __device__ __forceinline__ static void red(uint32_t* p, uint32_t v) { atomicMax(p, v); }  // no return: a reduction
 };
@@ -246,7 +246,7 @@ struct OpBFS {  // CASMIN(Val(v), Val(u) + 1)
   static constexpr uint32_t kIdentity = kInf;
   static constexpr uint32_t kSource = 0;
   __device__ __forceinline__ static uint32_t relax(uint32_t sv, uint32_t) { return sv == kInf ? kInf : sv + 1; }
-  __device__ __forceinline__ static bool better(uint32_t a, uint32_t b) { return a < b; }
+  __host__ __device__ __forceinline__ static constexpr bool better(uint32_t a, uint32_t b) { return a < b; }
   __device__ __forceinline__ static uint32_t atomic(uint32_t* p, uint32_t v) { return atomicMin(p, v); }
   __device__ __forceinline__ static void red(uint32_t* p, uint32_t v) { atomicMin(p, v); }  // no return: a reduction
 };
@@ -258,7 +258,7 @@ struct OpSSNP {  // CASMIN(Val(v), max(Val(u), w))
   __device__ __forceinline__ static uint32_t relax(uint32_t sv, uint32_t w) {
     return sv == kInf ? kInf : (sv > w ? sv : w);
   }
-  __device__ __forceinline__ static bool better(uint32_t a, uint32_t b) { return a < b; }
+  __host__ __device__ __forceinline__ static constexpr bool better(uint32_t a, uint32_t b) { return a < b; }
   __device__ __forceinline__ static uint32_t atomic(uint32_t* p, uint32_t v) { return atomicMin(p, v); }
   __device__ __forceinline__ static void red(uint32_t* p, uint32_t v) { atomicMin(p, v); }  // no return: a reduction
 };
@@ -268,6 +268,15 @@ struct OpSSNP {  // CASMIN(Val(v), max(Val(u), w))
 // widths are kept as complements, since the widest path (max over paths of
 // the min weight) is the complement of the min over paths of the max
 // complemented weight.  Each lane relaxes with its own kind (kKind*).
+
+struct OpSSWPNot {  // SSWP on complemented widths: CASMIN(Val(v), max(Val(u), ~w))
+  static constexpr bool kLevels = false;
+  static constexpr uint32_t kIdentity = kInf;
+  static constexpr uint32_t kSource = 0;
+  __device__ __forceinline__ static uint32_t relax(uint32_t sv, uint32_t w) { return sv > ~w ? sv : ~w; }
+  __host__ __device__ __forceinline__ static constexpr bool better(uint32_t a, uint32_t b) { return a < b; }
+  __device__ __forceinline__ static void red(uint32_t* p, uint32_t v) { atomicMin(p, v); }
+};
 
 struct OpMixed {
   static constexpr bool kLevels = false;
@@ -283,7 +292,7 @@ struct OpMixed {
     const uint32_t x = kind == kKindMax ? w : ~w;
     return sv > x ? sv : x;
   }
-  __device__ __forceinline__ static bool better(uint32_t a, uint32_t b) { return a < b; }
+  __host__ __device__ __forceinline__ static constexpr bool better(uint32_t a, uint32_t b) { return a < b; }
   __device__ __forceinline__ static void red(uint32_t* p, uint32_t v) { atomicMin(p, v); }
 };
 

@@ -31,17 +31,18 @@ __global__ void __launch_bounds__(256) group_lanes_kernel(LanesArgs a) {
       w |= (any ? 1u : 0u) << (16u + l);
     }
     a.nflanes[k] = w;
-    if (a.iplanes) {
-      const uint64_t* mi = g.ipmask + (size_t)k * g.W;
-      uint32_t wi = 0;
-      for (uint32_t l = 0; l < a.nlanes; ++l) {
-        bool any, all;
-        window_any_all(mi, a.win[l], any, all);
-        wi |= (all ? 1u : 0u) << l;
-        wi |= (any ? 1u : 0u) << (16u + l);
-      }
-      a.iplanes[k] = wi;
+  }
+  if (!a.iplanes) return;
+  for (size_t k = blockIdx.x * (size_t)blockDim.x + threadIdx.x; k < g.pp.slots; k += (size_t)gridDim.x * blockDim.x) {
+    const uint64_t* m = g.ppmask + k * g.W;
+    uint32_t w = 0;
+    for (uint32_t l = 0; l < a.nlanes; ++l) {
+      bool any, all;
+      window_any_all(m, a.win[l], any, all);
+      w |= (all ? 1u : 0u) << l;
+      w |= (any ? 1u : 0u) << (16u + l);
     }
+    a.iplanes[k] = w;
   }
 }
 

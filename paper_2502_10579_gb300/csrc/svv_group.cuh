@@ -21,31 +21,11 @@
 #pragma once
 
 #include "svv_device.cuh"
+#include "svv_pull.cuh"
 #include "svv_push.cuh"
 #include "svv_team.cuh"
 
 namespace svv {
-
-// plain (L1-cacheable) load of a vertex's lane row; values only improve, so a
-// stale row gives worse candidates (see ld_val)
-template <int KL>
-__device__ __forceinline__ void ld_row(const uint32_t* p, uint32_t (&r)[KL]) {
-  if constexpr (KL == 2) {
-    const uint2 x = *reinterpret_cast<const uint2*>(p);
-    r[0] = x.x;
-    r[1] = x.y;
-  } else {
-    const uint4* q = reinterpret_cast<const uint4*>(p);
-#pragma unroll
-    for (int i = 0; i < KL / 4; ++i) {
-      const uint4 x = q[i];
-      r[4 * i] = x.x;
-      r[4 * i + 1] = x.y;
-      r[4 * i + 2] = x.z;
-      r[4 * i + 3] = x.w;
-    }
-  }
-}
 
 template <int KL>
 __device__ __forceinline__ void st_row(uint32_t* p, const uint32_t (&r)[KL]) {
@@ -68,10 +48,11 @@ __device__ __forceinline__ uint32_t lanes_of(uint32_t word) {
 
 // relax every lane of edge (u -> x, w) whose bit is set in `pm`, from the
 // source row `su`, against the target row at `xr`; returns true if some lane
-// of x was lowered (raised, for SSWP) by this edge
-template <class Op, int KL>
+// of x was lowered (raised, for SSWP) by this edge, and keeps the best of the
+// improved values in `key` (per lane, or one for all of them)
+template <class Op, int KL, int NK>
 __device__ __forceinline__ bool relax_lanes(const uint32_t (&su)[KL], uint32_t w, uint32_t pm, uint32_t* xr,
-                                            uint32_t kinds) {
+                                            uint32_t kinds, uint32_t (&key)[NK]) {
   uint32_t cur[KL];
   ld_row<KL>(xr, cur);
   bool imp = false;
@@ -81,12 +62,18 @@ __device__ __forceinline__ bool relax_lanes(const uint32_t (&su)[KL], uint32_t w
       const uint32_t cand = lane_relax<Op>(kinds, k, su[k], w);
       if (Op::better(cand, cur[k])) {
         Op::red(xr + k, cand);
+        key[NK > 1 ? k : 0] = max(key[NK > 1 ? k : 0], nf_key<Op>(cand));
         imp = true;
       }
     }
   }
   return imp;
 }
+
+template <bool B>
+struct Flag {
+  static constexpr bool value = B;
+};
 
 template <class Op, int KL, int PRED>
 __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned long long* stage) {
@@ -98,6 +85,33 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
   const unsigned gwarp = gtid >> 5, nwarps = nthreads >> 5;
   if (a.qerr && cta_read(a.qerr) != 0u) return false;
   PushStage st{stage + (threadIdx.x >> 5) * kStageUnits, 0u};
+  // The best improved value of every round goes to a ring as in the single
+  // solve: one for the whole group (a bound for each of its lanes), or one per
+  // lane for the two lanes of a mixed pair, whose values do not compare.
+  constexpr int NK = is_mixed<Op>::value && KL == 2 ? 2 : 1;
+  constexpr uint32_t kRing[2] = {0u, 8u};  // words of c->aux
+  __shared__ uint32_t s_changed, s_key[NK];  // this CTA's improvements of a pull round; its best value
+  if (threadIdx.x == 0) {
+    s_changed = 0u;
+    for (int k = 0; k < NK; ++k) s_key[k] = 0u;
+  }
+  uint32_t key[NK] = {};
+  auto fold_keys = [&]() {  // a CTA barrier comes between this and publish_keys
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+      const uint32_t m = __reduce_max_sync(kFullMask, key[k]);
+      if (lane == 0 && m) atomicMax(&s_key[k], m);
+      key[k] = 0u;
+    }
+  };
+  auto publish_keys = [&](uint32_t slot) {
+    if (threadIdx.x == 0)
+      for (int k = 0; k < NK; ++k)
+        if (s_key[k]) {
+          atomicMax(&c->aux[kRing[k] + slot], s_key[k]);
+          s_key[k] = 0u;
+        }
+  };
   const uint32_t allmask = (1u << a.nlanes) - 1u;  // lanes in use (nlanes <= KL <= 8)
 
   // round 0: starting rows and stamps
@@ -127,6 +141,8 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
       const bool mine = lane < a.nlanes;
       const uint32_t src = mine ? a.source[lane] : 0u;
       if (mine) a.val[(size_t)src * KL + lane] = Op::kSource;
+#pragma unroll
+      for (int k = 0; k < NK; ++k) key[k] = nf_key<Op>(Op::kSource);
       __syncwarp();
       bool push = false;
       uint32_t deg = 0;
@@ -152,7 +168,7 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
           x = e.x;
           uint32_t su[KL];
           ld_row<KL>(a.val + (size_t)u * KL, su);
-          if (relax_lanes<Op, KL>(su, e.y, pm, a.val + (size_t)x * KL, a.kinds) && atomicExch(a.stamp + x, 1u) != 1u) {
+          if (relax_lanes<Op, KL>(su, e.y, pm, a.val + (size_t)x * KL, a.kinds, key) && atomicExch(a.stamp + x, 1u) != 1u) {
             push = true;
             deg = __ldg(g.rp + x + 1) - __ldg(g.rp + x);
           }
@@ -161,7 +177,9 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
       stage_push_units(push, x, deg, a.cshift, st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
     }
   }
+  fold_keys();
   stage_flush_cta(st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
+  publish_keys(1u);
   if (!t.sync()) return false;
 
   unsigned long long relaxed = 0;
@@ -181,11 +199,13 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
     // pull round it is the n vertices stamped with `it`.  A large frontier is
     // pulled, a small one pushed.
     const bool dense = cta_read(&c->aux[3 + cur]) != 0u;
-    const bool can_pull = g.ifd != nullptr && a.pull_units != 0u;
+    const bool can_pull = g.pull != 0u && a.pull_units != 0u;
     const bool pull = can_pull && (dense ? (n > a.push_verts) : (n > a.pull_units));
     if (gtid == 0) {
       atomicExch(&c->qn[clr], 0u);
       atomicExch(&c->ticket[clr], 0u);
+#pragma unroll
+      for (int k = 0; k < NK; ++k) atomicExch(&c->aux[kRing[k] + clr], 0u);
       atomicExch(&c->aux[3 + nxt], pull ? 1u : 0u);
       atomicExch(&c->aux[6 + ((it + 1u) & 1u)], 0u);  // compaction counter of the next round
     }
@@ -194,207 +214,68 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
     unsigned* qn_out = &c->qn[nxt];
     const uint32_t stamp_next = it + 1u;
 
-    if (pull && KL == 2 && !Op::kLevels) {
-      // ---- pull round of a two-lane group, as the single solve's: a warp
-      // takes 128 consecutive in-edges (4 per lane), the lowest lane of each
-      // target's run loads the target's row alongside the source gathers, and
-      // lanes with the same target fold their candidates lane by lane
-      uint32_t changed = 0, scanned = 0;
-      const uint32_t EF = g.E - g.NF;
-      const uint32_t ntot = EF + g.NF;
-      const uint32_t nchunks = (ntot + 127u) >> 7;
-      for (uint32_t ch = gwarp; ch < nchunks; ch += nwarps) {
-        uint32_t d[4], src[4], w[4], pm[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t idx = (ch << 7) + 32u * j + lane;
-          d[j] = 0xFFFFFFFFu - lane;  // unique per lane when not live
-          src[j] = 0;
-          w[j] = 0;
-          pm[j] = 0;
-          if (idx < ntot) {
-            if (idx < EF) {
-              d[j] = ld_stream(g.ifd + idx);
-              const uint2 sw = ld_stream(g.ifcw + idx);
-              src[j] = sw.x;
-              w[j] = sw.y;
-              pm[j] = allmask;
-            } else {
-              const uint32_t k = idx - EF;
-              d[j] = ld_stream(g.ipd + k);
-              const uint2 sw = ld_stream(g.ipcw + k);
-              src[j] = sw.x;
-              w[j] = sw.y;
-              pm[j] = lanes_of<PRED>(ld_stream(a.iplanes + k)) & allmask;
-            }
-          }
-        }
-        uint2 tv[4];
-        unsigned lead = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const unsigned grp = __match_any_sync(kFullMask, d[j]);
-          const uint32_t idx = (ch << 7) + 32u * j + lane;
-          const bool ld = idx < ntot && lane == (unsigned)(__ffs(grp) - 1);
-          lead |= (ld ? 1u : 0u) << j;
-          tv[j] = ld ? *reinterpret_cast<const uint2*>(a.val + (size_t)d[j] * 2) : make_uint2(0u, 0u);
-        }
-        uint32_t c0[4], c1[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          c0[j] = c1[j] = Op::kIdentity;
-          if (pm[j]) {
-            const uint2 su = *reinterpret_cast<const uint2*>(a.val + (size_t)src[j] * 2);
-            if (pm[j] & 1u) c0[j] = lane_relax<Op>(a.kinds, 0, su.x, w[j]);
-            if (pm[j] & 2u) c1[j] = lane_relax<Op>(a.kinds, 1, su.y, w[j]);
-          }
-          scanned += __popc(__ballot_sync(kFullMask, pm[j] != 0u));
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const unsigned grp = __match_any_sync(kFullMask, d[j]);
-          const uint32_t b0 = Op::better(0u, 1u) ? __reduce_min_sync(grp, c0[j]) : __reduce_max_sync(grp, c0[j]);
-          const uint32_t b1 = Op::better(0u, 1u) ? __reduce_min_sync(grp, c1[j]) : __reduce_max_sync(grp, c1[j]);
-          if ((lead >> j) & 1u) {
-            uint32_t* xr = a.val + (size_t)d[j] * 2;
-            bool imp = false;
-            if (Op::better(b0, tv[j].x)) {
-              Op::red(xr, b0);
-              imp = true;
-            }
-            if (Op::better(b1, tv[j].y)) {
-              Op::red(xr + 1, b1);
-              imp = true;
-            }
-            if (imp) {
-              // a plain store, as in the other pull rounds
-              a.stamp[d[j]] = stamp_next;
-              ++changed;
-            }
-          }
-        }
-      }
-      if (lane == 0) relaxed += scanned;
-      const uint32_t wc = __reduce_add_sync(kFullMask, changed);
-      if (lane == 0 && wc) atomicAdd(qn_out, wc);
-      if (!t.sync()) return false;
-      continue;
-    }
     if (pull) {
-      // ---- pull round over the edge-flat transposed graph: each lane takes
-      // two in-edges per step, computes every lane's candidate from the
-      // source row, and lanes with the same target fold their candidates
-      // lane by lane; the lowest of them updates the target row.
-      uint32_t changed = 0, scanned = 0;
-      // BFS from the source: round `it` sets level `it` in every lane, so a
-      // target reached in all lanes skips its in-edges, and only sources
-      // reached before this round count (bottom-up BFS)
+      // ---- pull round: one pass over every in-edge, a (CUDA) lane per target
+      // and every value lane of the group in its registers
       const bool bottom_up = Op::kLevels && a.init == kInitSource;
-      const uint32_t EF = g.E - g.NF;
-      const uint32_t ntot = EF + g.NF;
-      const uint32_t nchunks = (ntot + 63u) >> 6;
-      // the next chunk's edges are loaded while this chunk's rows are gathered
-      auto load_chunk = [&](uint32_t ch, bool valid, uint32_t (&d)[2], uint32_t (&src)[2], uint32_t (&w)[2],
-                            uint32_t (&pm)[2]) {
+      uint32_t best[2];
+      cta_read2(&c->aux[kRing[0] + cur], &c->aux[kRing[NK - 1] + cur], best[0], best[1]);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const uint32_t idx = (ch << 6) + 32u * j + lane;
-          d[j] = 0xFFFFFFFFu - lane;  // unique per lane when not live
-          src[j] = 0;
-          w[j] = 0;
-          pm[j] = 0;
-          if (valid && idx < ntot) {
-            if (idx < EF) {
-              d[j] = ld_stream(g.ifd + idx);
-              const uint2 sw = ld_stream(g.ifcw + idx);
-              src[j] = sw.x;
-              w[j] = sw.y;
-              pm[j] = allmask;
-            } else {
-              const uint32_t k = idx - EF;
-              d[j] = ld_stream(g.ipd + k);
-              const uint2 sw = ld_stream(g.ipcw + k);
-              src[j] = sw.x;
-              w[j] = sw.y;
-              pm[j] = lanes_of<PRED>(ld_stream(a.iplanes + k)) & allmask;
-            }
-          }
-        }
+      for (int k = 0; k < 2; ++k) best[k] = Op::better(0u, 1u) ? ~best[k] : best[k];
+      // three or more lanes of several types have no common bound
+      if (is_mixed<Op>::value && NK == 1) best[0] = Op::kSource;
+      PullRound pr{a.val, a.stamp, stamp_next, it, allmask, a.kinds, bottom_up ? it - 1u : best[0], bottom_up};
+      uint32_t changed = 0;
+      auto pull_rows = [&](auto desc) {  // every value lane of pr.mask at once
+        constexpr bool kDesc = decltype(desc)::value;
+        changed += pull_items<Op, KL, KL, true, kDesc>(g.pf, pr, gwarp, nwarps, lane, relaxed, key[0],
+                                                       [](size_t) { return ~0u; });
+        changed += pull_items<Op, KL, KL, false, kDesc>(
+            g.pp, pr, gwarp, nwarps, lane, relaxed, key[0],
+            [&](size_t slot) { return lanes_of<PRED>(ld_stream(a.iplanes + slot)); });
       };
-      uint32_t d[2], src[2], w[2], pm[2];
-      load_chunk(gwarp, gwarp < nchunks, d, src, w, pm);
-      for (uint32_t ch = gwarp; ch < nchunks; ch += nwarps) {
-        uint32_t dn[2], srcn[2], wn[2], pmn[2];
-        const bool more = ch + nwarps < nchunks;
-        load_chunk(more ? ch + nwarps : ch, more, dn, srcn, wn, pmn);
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const uint32_t idx = (ch << 6) + 32u * j + lane;
-          if (bottom_up && pm[j]) {
-            uint32_t dv[KL];
-            ld_row<KL>(a.val + (size_t)d[j] * KL, dv);
-            uint32_t open = 0;
-#pragma unroll
-            for (int k = 0; k < KL; ++k) open |= (dv[k] == kInf ? 1u : 0u) << k;
-            pm[j] &= open;
+      if constexpr (is_mixed<Op>::value && KL == 2) {
+        // two types: a pass per value lane, as in the single solve of its type
+        for (uint32_t k = 0; k < a.nlanes; ++k) {
+          pr.val = a.val + k;
+          pr.mask = 1u;
+          pr.best = best[k];
+          uint32_t lkey = 0;
+          auto pull_lane = [&](auto op, auto desc) {
+            using LaneOp = decltype(op);
+            constexpr bool kDesc = decltype(desc)::value;
+            changed += pull_items<LaneOp, 1, 2, true, kDesc>(g.pf, pr, gwarp, nwarps, lane, relaxed, lkey,
+                                                             [](size_t) { return 1u; });
+            changed += pull_items<LaneOp, 1, 2, false, kDesc>(
+                g.pp, pr, gwarp, nwarps, lane, relaxed, lkey,
+                [&](size_t slot) { return (lanes_of<PRED>(ld_stream(a.iplanes + slot)) >> k) & 1u; });
+          };
+          switch ((a.kinds >> (2u * k)) & 3u) {
+            case kKindSum: pull_lane(OpSSSP{}, Flag<false>{}); break;
+            case kKindHop: pull_lane(OpBFS{}, Flag<false>{}); break;
+            case kKindMax: pull_lane(OpSSNP{}, Flag<false>{}); break;
+            default: pull_lane(OpSSWPNot{}, Flag<true>{}); break;
           }
-          // the lowest lane of the target's run loads the target's row
-          // alongside the source row, not after the fold
-          const unsigned grp = __match_any_sync(kFullMask, d[j]);
-          const bool leader = idx < ntot && lane == (unsigned)(__ffs(grp) - 1);
-          uint32_t* xr = a.val + (size_t)d[j] * KL;
-          uint32_t cv[KL];
-          if (leader) {
-            ld_row<KL>(xr, cv);
-          } else {
-#pragma unroll
-            for (int k = 0; k < KL; ++k) cv[k] = Op::kIdentity;
-          }
-          uint32_t cand[KL];
-#pragma unroll
-          for (int k = 0; k < KL; ++k) cand[k] = Op::kIdentity;
-          if (pm[j]) {
-            uint32_t su[KL];
-            ld_row<KL>(a.val + (size_t)src[j] * KL, su);
-#pragma unroll
-            for (int k = 0; k < KL; ++k)
-              if (((pm[j] >> k) & 1u) && (!bottom_up || su[k] < it)) cand[k] = lane_relax<Op>(a.kinds, k, su[k], w[j]);
-          }
-          scanned += __popc(__ballot_sync(kFullMask, pm[j] != 0u));
-          uint32_t best[KL];
-#pragma unroll
-          for (int k = 0; k < KL; ++k)
-            best[k] = Op::better(0u, 1u) ? __reduce_min_sync(grp, cand[k]) : __reduce_max_sync(grp, cand[k]);
-          const bool any = __reduce_or_sync(grp, pm[j]) != 0u;
-          if (leader && any) {
-            bool imp = false;
-#pragma unroll
-            for (int k = 0; k < KL; ++k) {
-              if (Op::better(best[k], cv[k])) {
-                Op::red(xr + k, best[k]);
-                imp = true;
-              }
-            }
-            if (imp) {
-              // a plain store: the next round finds the changed vertices from
-              // the stamps, so `changed` only needs to be zero exactly when
-              // nothing changed
-              a.stamp[d[j]] = stamp_next;
-              ++changed;
-            }
-          }
+          if (NK > 1) key[NK > 1 && k ? 1 : 0] = lkey;
         }
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          d[j] = dn[j];
-          src[j] = srcn[j];
-          w[j] = wn[j];
-          pm[j] = pmn[j];
-        }
+      } else if constexpr (is_mixed<Op>::value) {
+        // widest-path lanes take the in-edges from the heaviest down, the
+        // others from the lightest up
+        uint32_t down = 0;
+        for (uint32_t k = 0; k < a.nlanes; ++k)
+          if (((a.kinds >> (2u * k)) & 3u) == kKindMaxNot) down |= 1u << k;
+        pr.mask = allmask & ~down;
+        if (pr.mask) pull_rows(Flag<false>{});
+        pr.mask = allmask & down;
+        if (pr.mask) pull_rows(Flag<true>{});
+      } else {
+        pull_rows(Flag<!Op::better(0u, 1u)>{});
       }
-      if (lane == 0) relaxed += scanned;
-      const uint32_t wc = __reduce_add_sync(kFullMask, changed);
-      if (lane == 0 && wc) atomicAdd(qn_out, wc);
+      fold_changes(changed, &s_changed, lane);
+      fold_keys();
+      __syncthreads();
+      publish_changes(&s_changed, qn_out);
+      publish_keys(nxt);
       if (!t.sync()) return false;
       continue;
     }
@@ -464,7 +345,7 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
               for (int k = 0; k < KL; ++k)
                 if (su[k] >= it) pm &= ~(1u << k);
             }
-            if (pm && relax_lanes<Op, KL>(su, ew.y, pm, a.val + (size_t)x * KL, a.kinds) &&
+            if (pm && relax_lanes<Op, KL>(su, ew.y, pm, a.val + (size_t)x * KL, a.kinds, key) &&
                 atomicExch(a.stamp + x, stamp_next) != stamp_next) {
               push = true;
               deg = __ldg(g.rp + x + 1) - __ldg(g.rp + x);
@@ -474,7 +355,9 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
         stage_push_units(push, x, deg, a.cshift, st, qout, qn_out, a.qcap, c, a.qerr, lane);
       }
     }
+    fold_keys();
     stage_flush_cta(st, qout, qn_out, a.qcap, c, a.qerr, lane);
+    publish_keys(nxt);
     if (!t.sync()) return false;
   }
   if (lane == 0 && relaxed) atomicAdd(&c->relaxed, relaxed);

@@ -23,7 +23,7 @@ svv_status ensure_group(svv_ctx* c) {
   svv_status st;
   if ((st = alloc_n(c, c->group_bufs, V * kGroupMax, &c->gcap)) ||
       (st = alloc_n(c, c->group_bufs, V * kGroupMax, &c->gcup)) || (st = alloc_n(c, c->group_bufs, NF, &c->gnfl)) ||
-      (st = alloc_n(c, c->group_bufs, NF, &c->gipl)) || (st = alloc_n(c, c->group_bufs, 1, &c->gerr))) {
+      (st = alloc_n(c, c->group_bufs, std::max<uint64_t>(c->g.pp.slots, 1), &c->gipl)) || (st = alloc_n(c, c->group_bufs, 1, &c->gerr))) {
     free_group(c);
     return st;
   }
@@ -69,7 +69,7 @@ svv_status enqueue_group_bounds(svv_ctx* c, int t, const BatchInstance* inst, ui
   la.nlanes = n;
   for (uint32_t k = 0; k < n; ++k) la.win[k] = Window{inst[k].wb, inst[k].wl};
   la.nflanes = c->gnfl;
-  la.iplanes = c->g.ifd ? c->gipl : nullptr;
+  la.iplanes = c->g.pull ? c->gipl : nullptr;
   if ((e = launch_group_lanes(la, s)) != cudaSuccess) return cuda_fail(c, e, "launch lane words");
 
   const SolveArgs base = solve_base(c, 0, 1, t, kn);
@@ -94,7 +94,7 @@ svv_status enqueue_group_bounds(svv_ctx* c, int t, const BatchInstance* inst, ui
   uint32_t pull_u[2] = {0, 0}, push_v[2] = {0, 0};
   for (int i = 0; i < 2; ++i) {
     const uint32_t pct = c->group_pull_pct[i];
-    if (c->g.ifd && pct && pct < 100) {
+    if (c->g.pull && pct && pct < 100) {
       const uint64_t all_units = (uint64_t)c->g.V + (c->g.E >> kn.solve_cs);
       pull_u[i] = (uint32_t)std::max<uint64_t>(1, all_units * pct / 100);
       push_v[i] = (uint32_t)std::max<uint64_t>(1, (uint64_t)c->g.V * pct / 100);

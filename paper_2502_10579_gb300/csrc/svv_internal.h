@@ -40,6 +40,20 @@ struct alignas(128) TeamCtl {
 };
 static_assert(sizeof(TeamCtl) % 128 == 0, "TeamCtl must be cache-line sized");
 
+// In-edges for pull rounds, a lane per target (built by svv_layout.cu): slice
+// s holds the targets tgt[32 s .. 32 s + 31] (kNone: no target); an item is
+// {first row of 32 slots, slice << 4 | (steps - 1)}, and step k of it is the 32
+// slots {source, weight} of row first + k, one per target.  The first nhub
+// slices hold one target each, its in-edges over all lanes.
+constexpr uint32_t kItemSteps = 16;
+struct PullGraph {
+  const uint2* items;
+  const uint32_t* tgt;
+  const uint2* cw;
+  uint32_t nitems, nhub;
+  uint64_t slots;
+};
+
 // Resident versioned graph (Section 4.1 layout, reordered at load):
 // row v holds edges [rp[v], rp[v+1]); the first (rp[v+1]-rp[v]) -
 // (nfp[v+1]-nfp[v]) of them are present in all S snapshots and carry no
@@ -55,16 +69,12 @@ struct DevGraph {
   const uint64_t* nfmask;   // [NF*W]
   const uint32_t* nfsrc;    // [NF]
   const uint2* nfcw;        // [NF]
-  // Transposed graph for pull rounds, edge-flat (may be absent: ifd ==
-  // nullptr).  The E-NF in-edges present in all S snapshots, sorted by
-  // target: ifd[i] is the target, ifcw[i] (source, weight).  The NF partial
-  // in-edges, sorted by target, in their own arrays with W mask words each
-  // at ipmask[k*W].  A pull pass streams both with no row lookups.
-  const uint32_t* ifd;      // [E-NF]
-  const uint2* ifcw;        // [E-NF]
-  const uint32_t* ipd;      // [NF]
-  const uint2* ipcw;        // [NF]
-  const uint64_t* ipmask;   // [NF*W]
+  // Transposed graph for pull rounds (pull == 0: not built): the E-NF in-edges
+  // present in all S snapshots, and the NF partial in-edges with W mask words
+  // per slot (0 in padding slots)
+  uint32_t pull;
+  PullGraph pf, pp;
+  const uint64_t* ppmask;   // [pp.slots*W]
 };
 
 struct Window {
@@ -286,7 +296,7 @@ struct GroupArgs {
   const uint32_t* base;            // kInitSeed: the intersection rows [V * KL]
   uint32_t* val;                   // [V * KL] result rows
   const uint32_t* nflanes;         // [NF] lane word of each partial edge, row order
-  const uint32_t* iplanes;         // [NF] lane word of each partial in-edge, transposed order
+  const uint32_t* iplanes;         // [pp.slots] lane word of each partial in-edge
   uint32_t* stamp;                 // [V]
   unsigned long long* q0;
   unsigned long long* q1;

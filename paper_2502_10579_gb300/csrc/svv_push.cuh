@@ -132,11 +132,17 @@ __device__ __forceinline__ void stage_flush_cta(PushStage& st, unsigned long lon
   __syncthreads();
 }
 
-// warp maximum of `x`; lane 0 folds it into *slot when any lane has `on` set
-__device__ __forceinline__ void warp_fold_max(bool on, uint32_t x, unsigned* slot, unsigned lane) {
-  if (__ballot_sync(kFullMask, on) == 0u) return;
-  const uint32_t m = __reduce_max_sync(kFullMask, on ? x : 0u);
-  if (lane == 0) atomicMax(slot, m);
+// Improvements counted by a pull round: every warp's into the CTA's word, then
+// (after a CTA barrier) the CTA's into the round's counter, one atomic per CTA.
+__device__ __forceinline__ void fold_changes(uint32_t changed, uint32_t* s_changed, unsigned lane) {
+  const uint32_t n = __reduce_add_sync(kFullMask, changed);
+  if (lane == 0 && n) atomicAdd(s_changed, n);
+}
+__device__ __forceinline__ void publish_changes(uint32_t* s_changed, unsigned* qn) {
+  if (threadIdx.x == 0 && *s_changed) {
+    atomicAdd(qn, *s_changed);
+    *s_changed = 0u;
+  }
 }
 
 }  // namespace svv

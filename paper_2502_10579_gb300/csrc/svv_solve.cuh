@@ -2,18 +2,11 @@
 #pragma once
 
 #include "svv_device.cuh"
+#include "svv_pull.cuh"
 #include "svv_push.cuh"
 #include "svv_team.cuh"
 
 namespace svv {
-
-
-// Near-far ordering key of a value: larger = closer to the source, so one
-// atomicMax per round finds the frontier's best value for both lattices.
-template <class Op>
-__device__ __forceinline__ uint32_t nf_key(uint32_t v) {
-  return Op::better(0u, 1u) ? ~v : v;
-}
 
 template <class Op, int PRED>
 __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long* stage) {
@@ -25,6 +18,8 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
   const unsigned gwarp = gtid >> 5, nwarps = nthreads >> 5;
   if (a.qerr && cta_read(a.qerr) != 0u) return false;
   PushStage st{stage + (threadIdx.x >> 5) * kStageUnits, 0u};
+  __shared__ uint32_t s_changed, s_key;  // this CTA's improvements of a round, and the best of them
+  if (threadIdx.x == 0) s_changed = s_key = 0u;
 
   // round 0: starting values and stamps
   if (a.init == kInitSource) {
@@ -45,6 +40,21 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
   if (!t.sync()) return false;
   if (a.trace && gtid == 0 && a.trace_cap) a.trace[0] = global_ns() & 0xFFFFFFFFFFull;
 
+  // the best value of each round's frontier goes to aux[0..2], a ring: every
+  // improvement of the round before counts, also those another lane beat
+  uint32_t key = 0;
+  auto fold_key = [&]() {  // a CTA barrier comes between this and publish_key
+    const uint32_t m = __reduce_max_sync(kFullMask, key);
+    if (lane == 0 && m) atomicMax(&s_key, m);
+    key = 0;
+  };
+  auto publish_key = [&](unsigned* slot) {
+    if (threadIdx.x == 0 && s_key) {
+      atomicMax(slot, s_key);
+      s_key = 0u;
+    }
+  };
+
   // round 0: first frontier (stamp 1, queue q1, count qn[1])
   if (a.init == kInitSource) {
     if (gwarp == 0) {
@@ -64,7 +74,7 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
     for (uint32_t k0 = gwarp * 32u; k0 < g.NF; k0 += nwarps * 32u) {
       const uint32_t k = k0 + lane;
       bool push = false;
-      uint32_t x = 0, deg = 0, cand = 0;
+      uint32_t x = 0, deg = 0;
       if (k < g.NF) {
         bool any, all;
         window_any_all(g.nfmask + (size_t)k * g.W, a.win, any, all);
@@ -72,9 +82,10 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
           const uint32_t u = __ldg(g.nfsrc + k);
           const uint2 e = __ldg(g.nfcw + k);
           x = e.x;
-          cand = Op::relax(ld_val(a.val + u), e.y);
+          const uint32_t cand = Op::relax(ld_val(a.val + u), e.y);
           if (Op::better(cand, ld_val(a.val + x))) {
             Op::red(a.val + x, cand);
+            key = max(key, nf_key<Op>(cand));
             const uint32_t r0 = __ldg(g.rp + x), r1 = __ldg(g.rp + x + 1);
             if (atomicExch(a.stamp + x, 1u) != 1u) {
               push = true;
@@ -84,10 +95,11 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
         }
       }
       stage_push_units(push, x, deg, a.cshift, st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
-      warp_fold_max(push, nf_key<Op>(cand), &c->aux[1], lane);
     }
   }
+  fold_key();
   stage_flush_cta(st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
+  publish_key(&c->aux[1]);
   if (!t.sync()) return false;
 
   unsigned long long relaxed = 0;
@@ -96,7 +108,7 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
     const uint32_t cur = it % 3u, nxt = (it + 1u) % 3u, clr = (it + 2u) % 3u;
     const bool far_on = a.delta != 0u;
     uint32_t n, slot;
-    cta_read2(&c->qn[cur], far_on ? &c->aux[cur] : nullptr, n, slot);
+    cta_read2(&c->qn[cur], &c->aux[cur], n, slot);
     if (a.trace && gtid == 0 && it < a.trace_cap) a.trace[it] = ((unsigned long long)n << 40) | (global_ns() & 0xFFFFFFFFFFull);
     if (n == 0u) break;
     if (it > a.maxit) {
@@ -109,7 +121,7 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
     // large frontier is pulled: every vertex takes the best candidate over
     // its in-edges (no queue, one atomic per chunk); a small one is pushed.
     const bool dense = cta_read(&c->aux[3 + cur]) != 0u;
-    const bool can_pull = g.ifd != nullptr && a.pull_units != 0u;
+    const bool can_pull = g.pull != 0u && a.pull_units != 0u;
     const bool pull = can_pull && (dense ? (n > a.push_verts) : (n > a.pull_units));
     if (gtid == 0) {
       atomicExch(&c->qn[clr], 0u);
@@ -124,92 +136,26 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
     const uint32_t stamp_next = it + 1u;
 
     if (pull) {
-      // ---- pull round: one pass over every in-edge, edge-flat.  A warp
-      // takes 128 consecutive in-edges (4 per lane, all loads issued before
-      // any reduction); lanes with the same target fold their candidates and
-      // the lowest of them updates the target.
-      uint32_t changed = 0, scanned = 0;
-      // BFS from the source: round `it` sets level `it` exactly when it only
-      // takes in-neighbours of level it-1; then every level already set is
-      // final and a visited target skips its in-edges (bottom-up BFS)
+      // ---- pull round: one pass over every in-edge, a lane per target
       const bool bottom_up = Op::kLevels && a.init == kInitSource;
-      const uint32_t EF = g.E - g.NF;
-      const uint32_t ntot = EF + ((PRED == kPredAll && a.skip_nf) ? 0u : g.NF);
-      const uint32_t nchunks = (ntot + 127u) >> 7;
-      for (uint32_t ch = gwarp; ch < nchunks; ch += nwarps) {
-        uint32_t d[4], src[4], w[4];
-        bool live[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t idx = (ch << 7) + 32u * j + lane;
-          live[j] = idx < ntot;
-          d[j] = 0xFFFFFFFFu - lane;  // unique per lane when not live
-          src[j] = 0;
-          w[j] = 0;
-          if (live[j]) d[j] = idx < EF ? ld_stream(g.ifd + idx) : ld_stream(g.ipd + (idx - EF));
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const uint32_t idx = (ch << 7) + 32u * j + lane;
-          if (live[j] && bottom_up && ld_val(a.val + d[j]) != kInf) live[j] = false;
-          if (live[j]) {
-            if (idx < EF) {
-              const uint2 sw = ld_stream(g.ifcw + idx);
-              src[j] = sw.x;
-              w[j] = sw.y;
-            } else {
-              const uint32_t k = idx - EF;
-              const uint64_t* m = g.ipmask + (size_t)k * g.W;
-              bool present;
-              if (PRED == kPredAll) present = window_all(m, a.win);
-              else if (PRED == kPredAny) present = window_any(m, a.win);
-              else present = mask_bit(m, a.bit);
-              const uint2 sw = ld_stream(g.ipcw + k);
-              src[j] = sw.x;
-              w[j] = sw.y;
-              live[j] = present;
-            }
-          }
-        }
-        // the lowest lane of each target's run loads the target's value now,
-        // alongside the source gathers, instead of after the fold
-        uint32_t cand[4], tv[4];
-        unsigned lead = 0;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const unsigned grp = __match_any_sync(kFullMask, d[j]);
-          const uint32_t idx = (ch << 7) + 32u * j + lane;
-          const bool ld = idx < ntot && lane == (unsigned)(__ffs(grp) - 1);
-          lead |= (ld ? 1u : 0u) << j;
-          tv[j] = ld ? ld_val(a.val + d[j]) : 0u;
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          cand[j] = Op::kIdentity;
-          if (live[j]) {
-            const uint32_t su = ld_val(a.val + src[j]);
-            if (!bottom_up || su < it) cand[j] = Op::relax(su, w[j]);
-          }
-          scanned += __popc(__ballot_sync(kFullMask, live[j]));
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const unsigned grp = __match_any_sync(kFullMask, d[j]);
-          const uint32_t best =
-              Op::better(0u, 1u) ? __reduce_min_sync(grp, cand[j]) : __reduce_max_sync(grp, cand[j]);
-          if (((lead >> j) & 1u) && Op::better(best, tv[j])) {
-            Op::red(a.val + d[j], best);
-            // a plain store: the next round finds the changed vertices from
-            // the stamps, so `changed` only needs to be zero exactly when
-            // nothing changed (it may count a vertex more than once)
-            a.stamp[d[j]] = stamp_next;
-            ++changed;
-          }
-        }
-      }
-      if (lane == 0) relaxed += scanned;
-      const uint32_t wc = __reduce_add_sync(kFullMask, changed);
-      if (lane == 0 && wc) atomicAdd(qn_out, wc);
+      constexpr bool kDesc = !Op::better(0u, 1u);
+      const PullRound pr{a.val, a.stamp, stamp_next, it, 1u, 0u,
+                         bottom_up ? it - 1u : (kDesc ? slot : ~slot), bottom_up};
+      uint32_t changed =
+          pull_items<Op, 1, 1, true, kDesc>(g.pf, pr, gwarp, nwarps, lane, relaxed, key, [](size_t) { return 1u; });
+      if (!(PRED == kPredAll && a.skip_nf))
+        changed += pull_items<Op, 1, 1, false, kDesc>(g.pp, pr, gwarp, nwarps, lane, relaxed, key,
+                                                   [&](size_t slot) -> uint32_t {
+                                                     const uint64_t* m = g.ppmask + slot * g.W;
+                                                     if (PRED == kPredAll) return window_all(m, a.win);
+                                                     if (PRED == kPredAny) return window_any(m, a.win);
+                                                     return mask_bit(m, a.bit);
+                                                   });
+      fold_changes(changed, &s_changed, lane);
+      fold_key();
+      __syncthreads();
+      publish_changes(&s_changed, qn_out);
+      publish_key(&c->aux[nxt]);
       if (!t.sync()) return false;
       continue;
     }
@@ -280,7 +226,7 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
       }
       if (far_on) {
         stage_push_units(defer, dv, ddeg, a.cshift, st, qout, qn_out, a.qcap, c, a.qerr, lane);
-        warp_fold_max(defer, nf_key<Op>(sv), &c->aux[nxt], lane);
+        if (defer) key = max(key, nf_key<Op>(sv));
       }
       const uint32_t incl = warp_incl_scan(cnt, lane);
       const uint32_t total = __shfl_sync(kFullMask, incl, 31);
@@ -332,7 +278,10 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           imp[j] = act[j] && Op::better(cand[j], curv[j]);
-          if (imp[j]) Op::red(a.val + x[j], cand[j]);
+          if (imp[j]) {
+            Op::red(a.val + x[j], cand[j]);
+            key = max(key, nf_key<Op>(cand[j]));
+          }
         }
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
@@ -346,13 +295,11 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
         }
         stage_push_units(push[0], x[0], deg[0], a.cshift, st, qout, qn_out, a.qcap, c, a.qerr, lane);
         stage_push_units(push[1], x[1], deg[1], a.cshift, st, qout, qn_out, a.qcap, c, a.qerr, lane);
-        if (far_on) {
-          const uint32_t k0v = push[0] ? nf_key<Op>(cand[0]) : 0u, k1v = push[1] ? nf_key<Op>(cand[1]) : 0u;
-          warp_fold_max(push[0] || push[1], max(k0v, k1v), &c->aux[nxt], lane);
-        }
       }
     }
+    fold_key();
     stage_flush_cta(st, qout, qn_out, a.qcap, c, a.qerr, lane);
+    publish_key(&c->aux[nxt]);
     if (!t.sync()) return false;
   }
   if (lane == 0 && relaxed) atomicAdd(&c->relaxed, relaxed);

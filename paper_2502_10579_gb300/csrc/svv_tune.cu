@@ -90,7 +90,7 @@ extern "C" svv_status svv_autotune(svv_ctx* c, svv_type type, uint32_t source, u
   const uint32_t cs0 = std::max<uint32_t>(c->solve_cs, 5u);
   if ((st = time_one(cur, &base_ms))) goto done;
   best_ms = base_ms;
-  if (c->g.ifd && (st = try_dim({0u, 5u, 10u, 15u, 25u, 40u}, [](Knobs& k, uint32_t v) { k.pull_pct = v; }))) goto done;
+  if (c->g.pull && (st = try_dim({0u, 5u, 10u, 15u, 25u, 40u}, [](Knobs& k, uint32_t v) { k.pull_pct = v; }))) goto done;
   if (t == 0 && (st = try_dim({0u, 250u, 1000u, 4000u}, [](Knobs& k, uint32_t v) { k.delta = v; }))) goto done;
   if (t == 1 && (st = try_dim({0u, 50u, 200u, 800u}, [](Knobs& k, uint32_t v) { k.delta = v; }))) goto done;
   if ((st = try_dim({cs0, cs0 + 1u}, [](Knobs& k, uint32_t v) { k.solve_cs = v; }))) goto done;
