@@ -460,11 +460,12 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
   g.W = W;
   g.E = E2;
   g.NF = NF;
-  uint32_t *d_rp, *d_nfp, *d_nfsrc;
+  uint32_t *d_rp, *d_nfsrc;
+  uint4* d_rowd;
   uint2 *d_cw, *d_nfcw;
   uint64_t* d_nfm;
   svv_status st;
-  if ((st = alloc_n(c, c->graph_bufs, (uint64_t)V + 1, &d_rp)) || (st = alloc_n(c, c->graph_bufs, (uint64_t)V + 1, &d_nfp)) ||
+  if ((st = alloc_n(c, c->graph_bufs, (uint64_t)V + 1, &d_rp)) || (st = alloc_n(c, c->graph_bufs, V, &d_rowd)) ||
       (st = alloc_n(c, c->graph_bufs, std::max<uint32_t>(E2, 1), &d_cw)) ||
       (st = alloc_n(c, c->graph_bufs, (uint64_t)std::max<uint32_t>(NF, 1) * W, &d_nfm)) ||
       (st = alloc_n(c, c->graph_bufs, std::max<uint32_t>(NF, 1), &d_nfsrc)) ||
@@ -473,7 +474,6 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
     return st;
   }
   cudaError_t e = cudaMemcpy(d_rp, rp.data(), rp.size() * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(d_nfp, nfp.data(), nfp.size() * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(d_cw, cw.data(), (size_t)E2 * 8, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(d_nfm, nfm.data(), (size_t)NF * W * 8, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(d_nfsrc, nfsrc.data(), (size_t)NF * 4, cudaMemcpyHostToDevice);
@@ -483,7 +483,7 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
     return cuda_fail(c, e, "uploading the graph");
   }
   g.rp = d_rp;
-  g.nfp = d_nfp;
+  g.rowd = d_rowd;
   g.cw = d_cw;
   g.nfmask = d_nfm;
   g.nfsrc = d_nfsrc;
@@ -514,7 +514,7 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
   c->pcap = (uint32_t)((uint64_t)V + (E2 >> 4) + 64);
   c->ecap = std::max<uint32_t>(E2, 1);
   c->g = g;
-  if (c->pull && (st = build_pull(c))) {
+  if ((st = build_rowd(c, nfp.data(), d_rowd)) || (c->pull && (st = build_pull(c)))) {
     free_graph(c);
     return st;
   }

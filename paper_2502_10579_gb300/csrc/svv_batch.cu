@@ -18,7 +18,7 @@
 
 namespace svv {
 
-constexpr int kBatchThreads = 512;
+constexpr int kBatchThreads = kStageThreads;
 constexpr uint32_t kNoInst = 0xFFFFFFFFu;
 constexpr uint32_t kSlab = 128;
 
@@ -61,12 +61,12 @@ __device__ uint32_t pick_instance(const BatchArgs& b) {
 // Out-of-line phase entry points: each phase keeps its own register
 // allocation instead of the sum of all of them inlined into one body.
 template <class Op, int PRED>
-__device__ __noinline__ bool solve_nl(const SolveArgs a, const Team t, unsigned long long* stage) {
+__device__ __noinline__ bool solve_nl(const SolveArgs a, const Team t, StageMem* stage) {
   return solve_team<Op, PRED>(a, t, stage);
 }
 __device__ __noinline__ bool qrs_nl(const QrsArgs a, const Team t) { return qrs_team(a, t); }
 template <class Op, int P, int K>
-__device__ __noinline__ bool relax_nl(const RelaxArgs a, const Team t, unsigned long long* stage) {
+__device__ __noinline__ bool relax_nl(const RelaxArgs a, const Team t, StageMem* stage) {
   return relax_team<Op, P, K>(a, t, stage);
 }
 __device__ __noinline__ void scatter_nl(const ScatterArgs a, const Team t, uint32_t* tile) {
@@ -75,7 +75,7 @@ __device__ __noinline__ void scatter_nl(const ScatterArgs a, const Team t, uint3
 
 template <class Op>
 __device__ bool run_instance(const BatchArgs& b, const BatchInstance& q, uint32_t i, const Team& t,
-                             const TeamScratch& sc, TeamCtl* tc, unsigned long long* stage, uint32_t* tile) {
+                             const TeamScratch& sc, TeamCtl* tc, StageMem* stage, uint32_t* tile) {
   SolveArgs a{};
   a.g = b.g;
   a.win = Window{q.wb, q.wl};
@@ -198,12 +198,14 @@ __device__ bool run_instance(const BatchArgs& b, const BatchInstance& q, uint32_
 }
 
 __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(BatchArgs b) {
-  __shared__ unsigned long long s_stage[(kBatchThreads / 32) * kStageUnits];
+  __shared__ StageMem s_stage;
   __shared__ uint32_t s_tile[kSlab * (kScatterTV + 1)];
   const unsigned team = blockIdx.x / b.team_blocks, rank = blockIdx.x % b.team_blocks;
   TeamCtl* tc = b.ctl + (size_t)team * kBatchCtl;
   const TeamScratch sc = b.scratch[team];
-  const Team base{tc, nullptr, b.team_blocks, rank, b.spin_ns};
+  __shared__ TeamBar s_bar;
+  const Team base{tc, nullptr, b.team_blocks, rank, b.spin_ns, &s_bar};
+  base.begin();
   for (;;) {
     if (rank == 0 && threadIdx.x == 0) {
       const uint32_t id = pick_instance(b);
@@ -219,10 +221,10 @@ __global__ void __launch_bounds__(kBatchThreads, 2) batch_kernel(BatchArgs b) {
     Team t = base;
     t.qerr = b.qerr + i;
     bool ok;
-    if (q.type == 0) ok = run_instance<OpSSSP>(b, q, i, t, sc, tc, s_stage, s_tile);
-    else if (q.type == 1) ok = run_instance<OpSSWP>(b, q, i, t, sc, tc, s_stage, s_tile);
-    else if (q.type == 3) ok = run_instance<OpSSNP>(b, q, i, t, sc, tc, s_stage, s_tile);
-    else ok = run_instance<OpBFS>(b, q, i, t, sc, tc, s_stage, s_tile);
+    if (q.type == 0) ok = run_instance<OpSSSP>(b, q, i, t, sc, tc, &s_stage, s_tile);
+    else if (q.type == 1) ok = run_instance<OpSSWP>(b, q, i, t, sc, tc, &s_stage, s_tile);
+    else if (q.type == 3) ok = run_instance<OpSSNP>(b, q, i, t, sc, tc, &s_stage, s_tile);
+    else ok = run_instance<OpBFS>(b, q, i, t, sc, tc, &s_stage, s_tile);
     if (rank == 0 && threadIdx.x == 0) {
       b.t_end[i] = global_ns();
       __threadfence_system();

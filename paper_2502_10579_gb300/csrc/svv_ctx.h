@@ -335,6 +335,7 @@ inline void slab_shape(uint32_t ls, uint32_t& P, uint32_t& K) {
   }
 }
 
+svv_status build_rowd(svv_ctx* c, const uint32_t* nfp, uint4* rowd);  // row descriptors (svv_layout.cu)
 svv_status build_pull(svv_ctx* c);  // the transposed graph (svv_layout.cu)
 
 // host helpers of the query pipeline (svv_api.cu)

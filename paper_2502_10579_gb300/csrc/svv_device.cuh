@@ -40,6 +40,11 @@ __device__ __forceinline__ uint2 ld_stream(const uint2* p) {
   return v;
 }
 
+// row of v as {begin, end}
+__device__ __forceinline__ uint2 ld_row_span(const DevGraph& g, uint32_t v) {
+  return __ldg(reinterpret_cast<const uint2*>(g.rowd + v));
+}
+
 __device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
   unsigned v;
   asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
@@ -57,16 +62,8 @@ __device__ __forceinline__ void set_err(TeamCtl* c, uint32_t* qerr, uint32_t cod
   if (qerr) atomicCAS(qerr, 0u, code);
 }
 
-__device__ __forceinline__ unsigned long long atom_add_acq_rel(unsigned long long* p, unsigned long long v) {
-  unsigned long long old;
-  asm volatile("atom.acq_rel.gpu.global.add.u64 %0, [%1], %2;" : "=l"(old) : "l"(p), "l"(v) : "memory");
-  return old;
-}
-
-__device__ __forceinline__ unsigned long long ld_acquire(const unsigned long long* p) {
-  unsigned long long v;
-  asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
+__device__ __forceinline__ void red_add_relaxed(unsigned long long* p, unsigned long long v) {
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" : : "l"(p), "l"(v) : "memory");
 }
 
 // Relaxed polls: an acquire load on every spin would also drop the SM's L1
@@ -86,65 +83,74 @@ __device__ __forceinline__ unsigned ld_relaxed(const unsigned* p) {
 
 __device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
-__device__ __forceinline__ void st_release(unsigned long long* p, unsigned long long v) {
-  asm volatile("st.release.gpu.global.u64 [%0], %1;" : : "l"(p), "l"(v) : "memory");
-}
-
-constexpr unsigned long long kGenErr = 1ull << 63;
-
 // ---------------------------------------------------------------------------
-// Team barrier over `nblocks` co-resident CTAs (cooperative launch), with a
-// bounded wait.  Arrivals are counted for the whole launch and never reset:
-// arrival number a belongs to barrier k = ceil(a / nblocks), and the CTA that
-// makes the count k * nblocks publishes k in `bar_gen` with a release store.
-// That last arriver also reads the team's error word (its acquire-release
-// add orders the read after every arrival, and so after every error set
-// before one) and publishes it in the same store, so every CTA learns of an
-// error from the one word it polls and they all leave together.  A CTA that
-// waits longer than `spin_ns`, or sees the error word set while waiting (a
-// CTA that timed out leaves without arriving), records the error and returns
-// false; every caller then leaves the kernel.
-__device__ __forceinline__ bool team_sync(TeamCtl* c, uint32_t* qerr, unsigned nblocks,
-                                          unsigned long long spin_ns) {
-  __shared__ int s_ok;
+// Team barrier over `nblocks` (< 2^15) co-resident CTAs (cooperative launch),
+// with a bounded wait.  An arrival adds 1 + (add << 16) to the barrier's word
+// with one release reduction, and every CTA polls that word until its low 16
+// bits show that all have arrived; the sum of the arrivals' `add` (the size of
+// the next round's frontier) is then in the rest of the word that was polled
+// anyway.  Barriers alternate between two words, so no CTA can add to a word
+// that another still polls; the words are never reset, and each CTA keeps what
+// they held after the barrier before (TeamBar), so the differences are exact
+// however often they wrap.  Arriving and polling on one word costs a fence, a
+// reduction's way to L2 and a load's way back; a last arriver that reads
+// counters and publishes them costs three more such trips (3.2 us a barrier
+// instead of about 2 on 456 CTAs).
+// A CTA that finds the team's error word set when it arrives adds an error
+// mark, so every CTA leaves after the same barrier.  A CTA that waits longer
+// than `spin_ns`, or sees the error word set while waiting (a CTA that timed
+// out leaves without arriving), records the error and returns false; every
+// caller then leaves the kernel.
+struct TeamBar {
+  unsigned long long word[2];  // what each word held after its last barrier
+  uint32_t k;                  // barriers passed
+};
+constexpr unsigned long long kBarErr = 1ull << 52;  // error mark: above any sum of `add` (< 2^33 << 16)
+
+__device__ __forceinline__ bool team_sync(TeamCtl* c, uint32_t* qerr, TeamBar* tb, unsigned nblocks,
+                                          unsigned long long spin_ns, uint32_t add, uint32_t& sum) {
+  __shared__ uint32_t s_ok, s_sum;
   __syncthreads();
   if (threadIdx.x == 0) {
     const uint32_t* ef = qerr ? qerr : &c->err;
-    const unsigned long long a = atom_add_acq_rel(&c->bar_count, 1ull) + 1ull;
-    const unsigned long long k = (a + nblocks - 1ull) / nblocks;
-    int ok = 1;
-    if (a == k * nblocks) {
-      const unsigned long long flag = ld_acquire(ef) != 0u ? kGenErr : 0ull;
-      st_release(&c->bar_gen, k | flag);
-      ok = flag == 0ull;
-    } else {
-      const unsigned long long t0 = global_ns();
-      unsigned polls = 0;
-      for (;;) {
-        const unsigned long long g = ld_relaxed(&c->bar_gen);
-        if ((g & ~kGenErr) >= k) {
-          fence_acq_rel();
-          ok = (g & kGenErr) == 0ull;
+    const uint32_t p = tb->k++ & 1u;
+    unsigned long long* w = &c->bar[p].v;
+    const unsigned long long before = tb->word[p];
+    unsigned long long mine = 1ull + ((unsigned long long)add << 16);
+    if (ld_relaxed(ef) != 0u) mine += kBarErr;
+    fence_acq_rel();
+    red_add_relaxed(w, mine);
+    const unsigned long long t0 = global_ns();
+    unsigned polls = 0;
+    uint32_t ok = 1;
+    unsigned long long d;
+    for (;;) {
+      const unsigned long long g = ld_relaxed(w);
+      d = g - before;
+      if ((d & 0xFFFFull) == nblocks) {
+        fence_acq_rel();
+        tb->word[p] = g;
+        break;
+      }
+      if ((++polls & 15u) == 0u) {
+        if (ld_relaxed(ef) != 0u) {
+          ok = 0;
           break;
         }
-        if ((++polls & 15u) == 0u) {
-          if (ld_relaxed(ef) != 0u) {
-            ok = 0;
-            break;
-          }
-          if (global_ns() - t0 > spin_ns) {
-            set_err(c, qerr, kErrTimeout);
-            ok = 0;
-            break;
-          }
+        if (global_ns() - t0 > spin_ns) {
+          set_err(c, qerr, kErrTimeout);
+          ok = 0;
+          break;
         }
-        if (polls > 64u) __nanosleep(64);
       }
+      if (polls > 64u) __nanosleep(64);
     }
-    s_ok = ok;
+    s_ok = ok && d < kBarErr;
+    s_sum = (uint32_t)(d >> 16);
   }
   __syncthreads();
-  return s_ok != 0;
+  sum = s_sum;
+  return s_ok != 0u;
 }
 
 // ---------------------------------------------------------------------------

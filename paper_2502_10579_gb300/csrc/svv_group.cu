@@ -16,7 +16,7 @@
 
 namespace svv {
 
-constexpr int kGroupThreads = 512;
+constexpr int kGroupThreads = kStageThreads;
 
 __global__ void __launch_bounds__(256) group_lanes_kernel(LanesArgs a) {
   const DevGraph& g = a.g;
@@ -49,9 +49,11 @@ __global__ void __launch_bounds__(256) group_lanes_kernel(LanesArgs a) {
 // two-lane groups fit 40 registers: 3 CTAs per SM, as the single solve
 template <class Op, int KL, int PRED>
 __global__ void __launch_bounds__(kGroupThreads, KL == 2 ? 3 : 2) group_solve_kernel(GroupArgs a) {
-  __shared__ unsigned long long s_stage[(kGroupThreads / 32) * kStageUnits];
-  const Team t{a.ctl, a.qerr, gridDim.x, blockIdx.x, a.spin_ns};
-  group_solve_team<Op, KL, PRED>(a, t, s_stage);
+  __shared__ StageMem s_stage;
+  __shared__ TeamBar s_bar;
+  const Team t{a.ctl, a.qerr, gridDim.x, blockIdx.x, a.spin_ns, &s_bar};
+  t.begin();
+  group_solve_team<Op, KL, PRED>(a, t, &s_stage);
 }
 
 // a thread per vertex: the lane rows of both bounds in, one word per lane and

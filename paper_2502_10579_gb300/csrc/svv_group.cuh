@@ -76,15 +76,17 @@ struct Flag {
 };
 
 template <class Op, int KL, int PRED>
-__device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned long long* stage) {
+__device__ bool group_solve_team(const GroupArgs& a, const Team& t, StageMem* stage) {
   const DevGraph& g = a.g;
   TeamCtl* c = a.ctl;
   const unsigned lane = threadIdx.x & 31u;
   const unsigned nthreads = t.nthreads();
   const unsigned gtid = t.tid();
-  const unsigned gwarp = gtid >> 5, nwarps = nthreads >> 5;
+  // neighbouring work goes to different SMs, so that a small round is spread
+  // over all of them
+  const unsigned gwarp = (threadIdx.x >> 5) * t.nblocks + t.rank, nwarps = nthreads >> 5;
   if (a.qerr && cta_read(a.qerr) != 0u) return false;
-  PushStage st{stage + (threadIdx.x >> 5) * kStageUnits, 0u};
+  PushStage st(stage);
   // The best improved value of every round goes to a ring as in the single
   // solve: one for the whole group (a bound for each of its lanes), or one per
   // lane for the two lanes of a mixed pair, whose values do not compare.
@@ -168,9 +170,10 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
           x = e.x;
           uint32_t su[KL];
           ld_row<KL>(a.val + (size_t)u * KL, su);
-          if (relax_lanes<Op, KL>(su, e.y, pm, a.val + (size_t)x * KL, a.kinds, key) && atomicExch(a.stamp + x, 1u) != 1u) {
-            push = true;
-            deg = __ldg(g.rp + x + 1) - __ldg(g.rp + x);
+          if (relax_lanes<Op, KL>(su, e.y, pm, a.val + (size_t)x * KL, a.kinds, key)) {
+            const uint2 r = ld_row_span(g, x);
+            push = atomicExch(a.stamp + x, 1u) != 1u;
+            deg = r.y - r.x;
           }
         }
       }
@@ -178,15 +181,16 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
     }
   }
   fold_keys();
-  stage_flush_cta(st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
+  uint32_t queued = stage_flush_cta(st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
   publish_keys(1u);
-  if (!t.sync()) return false;
+  uint32_t n = 0;  // the round's frontier: units, or vertices after a pull round
+  bool dense = false;
+  if (!t.sync(queued, n)) return false;
 
   unsigned long long relaxed = 0;
   uint32_t it = 1;
   for (;; ++it) {
     const uint32_t cur = it % 3u, nxt = (it + 1u) % 3u, clr = (it + 2u) % 3u;
-    uint32_t n = cta_read(&c->qn[cur]);
     if (a.trace && gtid == 0 && it < a.trace_cap)
       a.trace[it] = ((unsigned long long)n << 40) | (global_ns() & 0xFFFFFFFFFFull);
     if (n == 0u) break;
@@ -198,7 +202,6 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
     // After a push round the frontier is a unit queue of n units; after a
     // pull round it is the n vertices stamped with `it`.  A large frontier is
     // pulled, a small one pushed.
-    const bool dense = cta_read(&c->aux[3 + cur]) != 0u;
     const bool can_pull = g.pull != 0u && a.pull_units != 0u;
     const bool pull = can_pull && (dense ? (n > a.push_verts) : (n > a.pull_units));
     if (gtid == 0) {
@@ -206,7 +209,6 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
       atomicExch(&c->ticket[clr], 0u);
 #pragma unroll
       for (int k = 0; k < NK; ++k) atomicExch(&c->aux[kRing[k] + clr], 0u);
-      atomicExch(&c->aux[3 + nxt], pull ? 1u : 0u);
       atomicExch(&c->aux[6 + ((it + 1u) & 1u)], 0u);  // compaction counter of the next round
     }
     unsigned long long* qin = (it & 1u) ? a.q1 : a.q0;
@@ -274,9 +276,9 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
       fold_changes(changed, &s_changed, lane);
       fold_keys();
       __syncthreads();
-      publish_changes(&s_changed, qn_out);
       publish_keys(nxt);
-      if (!t.sync()) return false;
+      if (!t.sync(take_changes(&s_changed), n)) return false;
+      dense = true;
       continue;
     }
     if (dense) {
@@ -288,9 +290,10 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
         const uint32_t deg = take ? (__ldg(g.rp + v + 1) - __ldg(g.rp + v)) : 0u;
         stage_push_units(take, v, deg, a.cshift, st, qin, cnt_ctr, a.qcap, c, a.qerr, lane);
       }
-      stage_flush_cta(st, qin, cnt_ctr, a.qcap, c, a.qerr, lane);
-      if (!t.sync()) return false;
-      n = min(cta_read(cnt_ctr), a.qcap);
+      queued = stage_flush_cta(st, qin, cnt_ctr, a.qcap, c, a.qerr, lane);
+      if (!t.sync(queued, n)) return false;
+      n = min(n, a.qcap);
+      dense = false;
     }
 
     // ---- push round: a warp takes up to 32 units, prefix-sums their edge
@@ -304,10 +307,10 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
       if (lane < tk && ui < n) {
         const unsigned long long u = ld_cg(qin + ui);
         const uint32_t v = (uint32_t)u, ch = (uint32_t)(u >> 32);
-        const uint32_t r0 = __ldg(g.rp + v), r1 = __ldg(g.rp + v + 1);
-        const uint32_t nf0 = __ldg(g.nfp + v), nf1 = __ldg(g.nfp + v + 1);
-        fe = r1 - (nf1 - nf0);
-        nfb = nf0;
+        const uint4 rd = __ldg(g.rowd + v);
+        const uint32_t r0 = rd.x, r1 = rd.y;
+        fe = rd.z;
+        nfb = rd.w;
         vv = v;
         beg = r0 + (ch << a.cshift);
         const uint32_t end = min(r1, beg + (1u << a.cshift));
@@ -345,10 +348,10 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
               for (int k = 0; k < KL; ++k)
                 if (su[k] >= it) pm &= ~(1u << k);
             }
-            if (pm && relax_lanes<Op, KL>(su, ew.y, pm, a.val + (size_t)x * KL, a.kinds, key) &&
-                atomicExch(a.stamp + x, stamp_next) != stamp_next) {
-              push = true;
-              deg = __ldg(g.rp + x + 1) - __ldg(g.rp + x);
+            if (pm && relax_lanes<Op, KL>(su, ew.y, pm, a.val + (size_t)x * KL, a.kinds, key)) {
+              const uint2 r = ld_row_span(g, x);
+              push = atomicExch(a.stamp + x, stamp_next) != stamp_next;
+              deg = r.y - r.x;
             }
           }
         }
@@ -356,9 +359,9 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, unsigned lon
       }
     }
     fold_keys();
-    stage_flush_cta(st, qout, qn_out, a.qcap, c, a.qerr, lane);
+    queued = stage_flush_cta(st, qout, qn_out, a.qcap, c, a.qerr, lane);
     publish_keys(nxt);
-    if (!t.sync()) return false;
+    if (!t.sync(queued, n)) return false;
   }
   if (lane == 0 && relaxed) atomicAdd(&c->relaxed, relaxed);
   if (gtid == 0) c->iters = it - 1u;

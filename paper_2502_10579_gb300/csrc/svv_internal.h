@@ -24,10 +24,10 @@ enum Init : int { kInitSource = 0, kInitSeed = 1 };
 // it).  Fields live on separate 128-byte lines so the barrier counter does not
 // share a line with the counters that every warp hits.
 struct alignas(128) TeamCtl {
-  unsigned long long bar_count;  // arrivals since launch (never reset)
-  unsigned int pad0[30];
-  unsigned long long bar_gen;    // last released barrier | kGenErr
-  unsigned int pad1[30];
+  struct {
+    unsigned long long v;  // the barrier's word (team_sync), one for odd and one for even barriers
+    unsigned int pad[30];
+  } bar[2];
   unsigned int qn[3];      // frontier sizes, a ring over rounds
   unsigned int pad2[29];
   unsigned int ticket[3];  // work tickets, a ring over rounds
@@ -55,16 +55,17 @@ struct PullGraph {
 };
 
 // Resident versioned graph (Section 4.1 layout, reordered at load):
-// row v holds edges [rp[v], rp[v+1]); the first (rp[v+1]-rp[v]) -
-// (nfp[v+1]-nfp[v]) of them are present in all S snapshots and carry no
-// mask; the rest ("non-full") have W mask words at nfmask[(nfp[v]+j)*W].
+// row v holds edges [rp[v], rp[v+1]); the first of them are present in all S
+// snapshots and carry no mask; the rest ("non-full", from rowd[v].z on) have W
+// mask words each at nfmask[(rowd[v].w + j)*W].  A visited vertex reads rowd
+// (one 16-byte load); passes over all vertices in order read rp.
 // The non-full edges are also kept as a coordinate list (nfsrc, nfcw) in the
 // same order, for the seeding passes.
 struct DevGraph {
   uint32_t V, S, W;
   uint32_t E, NF;
   const uint32_t* rp;       // [V+1]
-  const uint32_t* nfp;      // [V+1]
+  const uint4* rowd;        // [V] {rp[v], rp[v+1], first non-full edge, its index in the non-full list}
   const uint2* cw;          // [E] (target, weight)
   const uint64_t* nfmask;   // [NF*W]
   const uint32_t* nfsrc;    // [NF]

@@ -201,10 +201,10 @@ __global__ void __launch_bounds__(256) list_kernel(DevGraph g, int part, uint2* 
       list[e] = make_uint2(w, (uint32_t)e);
       top = max(top, w);
     } else {
-      const uint32_t v = row_of(g, (uint32_t)e), nf0 = g.nfp[v];
-      if (e >= g.rp[v + 1] - (g.nfp[v + 1] - nf0)) continue;
+      const uint4 rd = g.rowd[row_of(g, (uint32_t)e)];
+      if (e >= rd.z) continue;
       const uint32_t w = g.cw[e].y;
-      list[e - nf0] = make_uint2(w, (uint32_t)e);
+      list[e - rd.w] = make_uint2(w, (uint32_t)e);
       top = max(top, w);
     }
   }
@@ -325,6 +325,23 @@ unsigned blocks_for(uint64_t n, unsigned per) {
 }
 
 }  // namespace
+
+__global__ void __launch_bounds__(256) rowd_kernel(const uint32_t* rp, const uint32_t* nfp, uint32_t V, uint4* rowd) {
+  for (size_t v = blockIdx.x * (size_t)blockDim.x + threadIdx.x; v < V; v += (size_t)gridDim.x * blockDim.x)
+    rowd[v] = make_uint4(rp[v], rp[v + 1], rp[v + 1] - (nfp[v + 1] - nfp[v]), nfp[v]);
+}
+
+// row descriptors from the row offsets and the (host) prefix counts of partial edges
+svv_status build_rowd(svv_ctx* c, const uint32_t* nfp, uint4* rowd) {
+  const uint32_t V = c->g.V;
+  cudaError_t e = cudaMemcpy(c->cur, nfp, ((size_t)V + 1) * 4, cudaMemcpyHostToDevice);  // cur holds 2V words
+  if (e == cudaSuccess) {
+    rowd_kernel<<<blocks_for(V, 1024), 256>>>(c->g.rp, c->cur, V, rowd);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+  return e == cudaSuccess ? SVV_OK : cuda_fail(c, e, "building the row descriptors");
+}
 
 // Build both halves of the transposed graph (edges present in every snapshot;
 // partial edges with their masks).  Runs on the legacy stream with the query

@@ -19,6 +19,7 @@
 #include "../../include/svv.h"
 #include "svv_device.cuh"
 #include "svv_push.cuh"
+#include "svv_team.cuh"
 
 namespace svv {
 namespace {
@@ -72,7 +73,10 @@ __global__ void __launch_bounds__(kNaThreads) noalloc_solve_kernel(NaArgs a) {
     const uint64_t r0 = __ldg(a.rp + v), r1 = __ldg(a.rp + v + 1);
     if (r1 < r0 || r1 > a.E || (v == 0 && r0 != 0) || (v + 1 == a.V && r1 != a.E)) set_err(c, a.qerr, kErrInput);
   }
-  if (!team_sync(c, a.qerr, gridDim.x, a.spin_ns)) return;
+  __shared__ TeamBar s_bar;
+  const Team t{c, a.qerr, gridDim.x, blockIdx.x, a.spin_ns, &s_bar};
+  t.begin();
+  if (!t.sync()) return;
 
   if (blockIdx.x == 0 && threadIdx.x < 32) {
     uint32_t deg = 0;
@@ -85,14 +89,14 @@ __global__ void __launch_bounds__(kNaThreads) noalloc_solve_kernel(NaArgs a) {
     }
     warp_push_units(lane == 0, a.source, deg, kNaChunkShift, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
   }
-  if (!team_sync(c, a.qerr, gridDim.x, a.spin_ns)) return;
+  if (!t.sync()) return;
 
   const uint32_t word = a.snap >> 6;
   const uint64_t bit = 1ull << (a.snap & 63u);
   uint32_t it = 1;
   for (;; ++it) {
     const uint32_t cur = it % 3u, nxt = (it + 1u) % 3u, clr = (it + 2u) % 3u;
-    uint32_t n = ld_acquire(&c->qn[cur]);
+    uint32_t n = cta_read(&c->qn[cur]);
     if (n == 0u) break;
     if (it > a.maxit) {
       if (gtid == 0) set_err(c, a.qerr, kErrTimeout);
@@ -164,7 +168,7 @@ __global__ void __launch_bounds__(kNaThreads) noalloc_solve_kernel(NaArgs a) {
         warp_push_units(push, x, deg, kNaChunkShift, qout, &c->qn[nxt], a.qcap, c, a.qerr, lane);
       }
     }
-    if (!team_sync(c, a.qerr, gridDim.x, a.spin_ns)) return;
+    if (!t.sync()) return;
   }
   if (gtid == 0) c->iters = it - 1u;
 }

@@ -27,7 +27,9 @@ namespace svv {
 constexpr int kQrsThreads = 512;
 
 __global__ void __launch_bounds__(kQrsThreads) qrs_kernel(QrsArgs a) {
-  const Team t{a.ctl, a.qerr, gridDim.x, blockIdx.x, a.spin_ns};
+  __shared__ TeamBar s_bar;
+  const Team t{a.ctl, a.qerr, gridDim.x, blockIdx.x, a.spin_ns, &s_bar};
+  t.begin();
   qrs_team(a, t);
 }
 

@@ -90,10 +90,10 @@ __device__ void qrs_walk(const QrsArgs& a, const Team& t, uint32_t NU, uint32_t 
       r = (uint32_t)u;
       const uint32_t ch = (uint32_t)(u >> 32);
       const uint32_t v = a.uv[r];
-      const uint32_t r0 = __ldg(g.rp + v), r1 = __ldg(g.rp + v + 1);
-      const uint32_t nf0 = __ldg(g.nfp + v), nf1 = __ldg(g.nfp + v + 1);
-      fe = r1 - (nf1 - nf0);
-      nfb = nf0;
+      const uint4 rd = __ldg(g.rowd + v);
+      const uint32_t r0 = rd.x, r1 = rd.y;
+      fe = rd.z;
+      nfb = rd.w;
       beg = r0 + (ch << a.cshift);
       const uint32_t end = min(r1, beg + (1u << a.cshift));
       cnt = end > beg ? end - beg : 0u;

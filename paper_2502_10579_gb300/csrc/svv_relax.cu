@@ -25,13 +25,15 @@
 
 namespace svv {
 
-constexpr int kRelaxThreads = 512;
+constexpr int kRelaxThreads = kStageThreads;
 
 template <class Op, int P, int K>
 __global__ void __launch_bounds__(kRelaxThreads, 2) relax_kernel(RelaxArgs a) {
-  __shared__ unsigned long long s_stage[(kRelaxThreads / 32) * kStageUnits];
-  const Team t{a.ctl, a.qerr, gridDim.x, blockIdx.x, a.spin_ns};
-  relax_team<Op, P, K>(a, t, s_stage);
+  __shared__ StageMem s_stage;
+  __shared__ TeamBar s_bar;
+  const Team t{a.ctl, a.qerr, gridDim.x, blockIdx.x, a.spin_ns, &s_bar};
+  t.begin();
+  relax_team<Op, P, K>(a, t, &s_stage);
 }
 
 // ---------------------------------------------------------------------------

@@ -16,15 +16,17 @@ __device__ __forceinline__ uint32_t relax_q(const RelaxArgs& a, bool q1, uint32_
 }
 
 template <class Op, int P, int K>
-__device__ bool relax_team(const RelaxArgs& a, const Team& t, unsigned long long* stage) {
+__device__ bool relax_team(const RelaxArgs& a, const Team& t, StageMem* stage) {
   const DevGraph& g = a.g;
   TeamCtl* c = a.ctl;
   const unsigned lane = threadIdx.x & 31u;
   const unsigned nthreads = t.nthreads();
   const unsigned gtid = t.tid();
-  const unsigned gwarp = gtid >> 5, nwarps = nthreads >> 5;
+  // neighbouring work goes to different SMs, so that a small round is spread
+  // over all of them
+  const unsigned gwarp = (threadIdx.x >> 5) * t.nblocks + t.rank, nwarps = nthreads >> 5;
   if (cta_read(a.qerr) != 0u) return false;
-  PushStage st{stage + (threadIdx.x >> 5) * kStageUnits, 0u};
+  PushStage st(stage);
   // rows [0, U0) are the first query's, [U0, U) a second query's (a.counts1)
   const uint32_t U0 = a.counts[0];
   const uint32_t U = U0 + (a.counts1 ? a.counts1[0] : 0u);
@@ -145,8 +147,9 @@ __device__ bool relax_team(const RelaxArgs& a, const Team& t, unsigned long long
       }
     }
   }
-  stage_flush_cta(st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
-  if (!t.sync()) return false;
+  uint32_t queued = stage_flush_cta(st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
+  uint32_t n = 0;  // units of the round
+  if (!t.sync(queued, n)) return false;
 
   // ---- rounds >= 1: Algorithm 2 while-loop over the frontier
   constexpr int G = 32 / P;
@@ -156,7 +159,6 @@ __device__ bool relax_team(const RelaxArgs& a, const Team& t, unsigned long long
   uint32_t it = 1;
   for (;; ++it) {
     const uint32_t cur = it % 3u, nxt = (it + 1u) % 3u, clr = (it + 2u) % 3u;
-    uint32_t n = cta_read(&c->qn[cur]);
     if (a.trace && gtid == 0 && it < a.trace_cap) a.trace[it] = ((unsigned long long)n << 40) | (global_ns() & 0xFFFFFFFFFFull);
     if (n == 0u) break;
     if (it > a.maxit) {
@@ -282,8 +284,8 @@ __device__ bool relax_team(const RelaxArgs& a, const Team& t, unsigned long long
         stage_push_units(push, pend_x, deg, a.cshift, st, qout, qn_out, a.qcap, c, a.qerr, lane);
       }
     }
-    stage_flush_cta(st, qout, qn_out, a.qcap, c, a.qerr, lane);
-    if (!t.sync()) return false;
+    queued = stage_flush_cta(st, qout, qn_out, a.qcap, c, a.qerr, lane);
+    if (!t.sync(queued, n)) return false;
   }
   if (gl == 0 && relaxed) atomicAdd(&c->relaxed, relaxed);
   if (gtid == 0) c->iters = it - 1u;

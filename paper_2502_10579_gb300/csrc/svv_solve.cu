@@ -18,13 +18,15 @@
 
 namespace svv {
 
-constexpr int kSolveThreads = 512;
+constexpr int kSolveThreads = kStageThreads;
 
 template <class Op, int PRED>
 __global__ void __launch_bounds__(kSolveThreads, 3) solve_kernel(SolveArgs a) {
-  __shared__ unsigned long long s_stage[(kSolveThreads / 32) * kStageUnits];
-  const Team t{a.ctl, a.qerr, gridDim.x, blockIdx.x, a.spin_ns};
-  solve_team<Op, PRED>(a, t, s_stage);
+  __shared__ StageMem s_stage;
+  __shared__ TeamBar s_bar;
+  const Team t{a.ctl, a.qerr, gridDim.x, blockIdx.x, a.spin_ns, &s_bar};
+  t.begin();
+  solve_team<Op, PRED>(a, t, &s_stage);
 }
 
 template <class Op, int PRED>

@@ -9,15 +9,17 @@
 namespace svv {
 
 template <class Op, int PRED>
-__device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long* stage) {
+__device__ bool solve_team(const SolveArgs& a, const Team& t, StageMem* stage) {
   const DevGraph& g = a.g;
   TeamCtl* c = a.ctl;
   const unsigned lane = threadIdx.x & 31u;
   const unsigned nthreads = t.nthreads();
   const unsigned gtid = t.tid();
-  const unsigned gwarp = gtid >> 5, nwarps = nthreads >> 5;
+  // neighbouring work goes to different SMs, so that a small round is spread
+  // over all of them
+  const unsigned gwarp = (threadIdx.x >> 5) * t.nblocks + t.rank, nwarps = nthreads >> 5;
   if (a.qerr && cta_read(a.qerr) != 0u) return false;
-  PushStage st{stage + (threadIdx.x >> 5) * kStageUnits, 0u};
+  PushStage st(stage);
   __shared__ uint32_t s_changed, s_key;  // this CTA's improvements of a round, and the best of them
   if (threadIdx.x == 0) s_changed = s_key = 0u;
 
@@ -86,10 +88,10 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
           if (Op::better(cand, ld_val(a.val + x))) {
             Op::red(a.val + x, cand);
             key = max(key, nf_key<Op>(cand));
-            const uint32_t r0 = __ldg(g.rp + x), r1 = __ldg(g.rp + x + 1);
+            const uint2 r = ld_row_span(g, x);
             if (atomicExch(a.stamp + x, 1u) != 1u) {
               push = true;
-              deg = r1 - r0;
+              deg = r.y - r.x;
             }
           }
         }
@@ -98,17 +100,17 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
     }
   }
   fold_key();
-  stage_flush_cta(st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
+  uint32_t queued = stage_flush_cta(st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
   publish_key(&c->aux[1]);
-  if (!t.sync()) return false;
+  uint32_t n = 0;  // the round's frontier: units, or vertices after a pull round
+  bool dense = false;
+  if (!t.sync(queued, n)) return false;
 
   unsigned long long relaxed = 0;
   uint32_t it = 1;
   for (;; ++it) {
     const uint32_t cur = it % 3u, nxt = (it + 1u) % 3u, clr = (it + 2u) % 3u;
     const bool far_on = a.delta != 0u;
-    uint32_t n, slot;
-    cta_read2(&c->qn[cur], &c->aux[cur], n, slot);
     if (a.trace && gtid == 0 && it < a.trace_cap) a.trace[it] = ((unsigned long long)n << 40) | (global_ns() & 0xFFFFFFFFFFull);
     if (n == 0u) break;
     if (it > a.maxit) {
@@ -120,14 +122,12 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
     // n units; after a pull round it is the n vertices stamped with `it`.  A
     // large frontier is pulled: every vertex takes the best candidate over
     // its in-edges (no queue, one atomic per chunk); a small one is pushed.
-    const bool dense = cta_read(&c->aux[3 + cur]) != 0u;
     const bool can_pull = g.pull != 0u && a.pull_units != 0u;
     const bool pull = can_pull && (dense ? (n > a.push_verts) : (n > a.pull_units));
     if (gtid == 0) {
       atomicExch(&c->qn[clr], 0u);
       atomicExch(&c->ticket[clr], 0u);
       atomicExch(&c->aux[clr], 0u);
-      atomicExch(&c->aux[3 + nxt], pull ? 1u : 0u);
       atomicExch(&c->aux[6 + ((it + 1u) & 1u)], 0u);  // compaction counter of the next round
     }
     unsigned long long* qin = (it & 1u) ? a.q1 : a.q0;
@@ -138,6 +138,7 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
     if (pull) {
       // ---- pull round: one pass over every in-edge, a lane per target
       const bool bottom_up = Op::kLevels && a.init == kInitSource;
+      const uint32_t slot = cta_read(&c->aux[cur]);
       constexpr bool kDesc = !Op::better(0u, 1u);
       const PullRound pr{a.val, a.stamp, stamp_next, it, 1u, 0u,
                          bottom_up ? it - 1u : (kDesc ? slot : ~slot), bottom_up};
@@ -154,9 +155,9 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
       fold_changes(changed, &s_changed, lane);
       fold_key();
       __syncthreads();
-      publish_changes(&s_changed, qn_out);
       publish_key(&c->aux[nxt]);
-      if (!t.sync()) return false;
+      if (!t.sync(take_changes(&s_changed), n)) return false;
+      dense = true;
       continue;
     }
     if (dense) {
@@ -168,15 +169,17 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
         const uint32_t deg = take ? (__ldg(g.rp + v + 1) - __ldg(g.rp + v)) : 0u;
         stage_push_units(take, v, deg, a.cshift, st, qin, cnt_ctr, a.qcap, c, a.qerr, lane);
       }
-      stage_flush_cta(st, qin, cnt_ctr, a.qcap, c, a.qerr, lane);
-      if (!t.sync()) return false;
-      n = min(cta_read(cnt_ctr), a.qcap);
+      queued = stage_flush_cta(st, qin, cnt_ctr, a.qcap, c, a.qerr, lane);
+      if (!t.sync(queued, n)) return false;
+      n = min(n, a.qcap);
+      dense = false;
     }
     // near-far: relax only units whose value is within delta of the best
     // value queued for this round (that unit itself always qualifies, so every
     // round makes progress); the others are queued again unchanged
     uint32_t bound = 0;
     if (far_on) {
+      const uint32_t slot = cta_read(&c->aux[cur]);
       if (Op::better(0u, 1u)) {
         const uint32_t best = ~slot;
         bound = best > kInf - a.delta ? kInf : best + a.delta;
@@ -197,10 +200,10 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
       if (lane < tk && ui < n) {
         const unsigned long long u = ld_cg(qin + ui);
         const uint32_t v = (uint32_t)u, ch = (uint32_t)(u >> 32);
-        const uint32_t r0 = __ldg(g.rp + v), r1 = __ldg(g.rp + v + 1);
-        const uint32_t nf0 = __ldg(g.nfp + v), nf1 = __ldg(g.nfp + v + 1);
-        fe = r1 - (nf1 - nf0);
-        nfb = nf0;
+        const uint4 rd = __ldg(g.rowd + v);
+        const uint32_t r0 = rd.x, r1 = rd.y;
+        fe = rd.z;
+        nfb = rd.w;
         beg = r0 + (ch << a.cshift);
         uint32_t end = min(r1, beg + (1u << a.cshift));
         if (PRED == kPredAll && a.skip_nf) end = min(end, fe);
@@ -286,10 +289,10 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
           if (imp[j]) {
-            const uint32_t r0 = __ldg(g.rp + x[j]), r1 = __ldg(g.rp + x[j] + 1);
+            const uint2 r = ld_row_span(g, x[j]);
             if (atomicExch(a.stamp + x[j], stamp_next) != stamp_next) {
               push[j] = true;
-              deg[j] = r1 - r0;
+              deg[j] = r.y - r.x;
             }
           }
         }
@@ -298,9 +301,9 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, unsigned long long
       }
     }
     fold_key();
-    stage_flush_cta(st, qout, qn_out, a.qcap, c, a.qerr, lane);
+    queued = stage_flush_cta(st, qout, qn_out, a.qcap, c, a.qerr, lane);
     publish_key(&c->aux[nxt]);
-    if (!t.sync()) return false;
+    if (!t.sync(queued, n)) return false;
   }
   if (lane == 0 && relaxed) atomicAdd(&c->relaxed, relaxed);
   if (gtid == 0) c->iters = it - 1u;

@@ -92,3 +92,29 @@ def test_source_far_from_targets(svv):
         ctx.load_log(log)
         for t in range(4):
             np.testing.assert_array_equal(svv.to_u32(ctx.query(t, 2990, 3, 50)), oracle.query(log, t, 2990, 3, 50))
+
+
+@pytest.mark.parametrize("blocks", [1, 0])
+def test_rounds_that_queue_mostly_hubs(svv, blocks):
+    """Every vertex has 34 work units, so one push round lists far more vertices
+    per CTA than its hub list holds (blocks_per_sm = 1), or about as many."""
+    rng = np.random.default_rng(5)
+    V, d = 24000, 544
+    n = V * d
+    log = EdgeLog(V=V, S=2, src=np.repeat(np.arange(V, dtype=np.uint32), d),
+                  dst=rng.integers(0, V, size=n).astype(np.uint32), w=rng.integers(1, 1000, size=n).astype(np.uint32),
+                  add_off=np.array([0, n, n]), del_off=np.array([0, 0, 100]), del_ids=np.arange(100),
+                  t_add=np.zeros(n, np.uint32), t_del=np.where(np.arange(n) < 100, 1, 2).astype(np.uint32), meta={})
+    with svv.Context(0) as ctx:
+        ctx.set_tuning("solve_chunk", 16)
+        ctx.set_tuning("pull_pct", 0)
+        ctx.set_tuning("group_pull_pct", 0)
+        ctx.set_tuning("blocks_per_sm", blocks)
+        ctx.load_log(log)
+        want = [oracle.query(log, t, 0, 0, 2) for t in (0, 2)]
+        for t, w in zip((0, 2), want):
+            np.testing.assert_array_equal(svv.to_u32(ctx.query(t, 0, 0, 2)), w)
+        ctx.set_tuning("batch_mode", 2)
+        outs, _ = ctx.query_batch([(0, 0, 0, 2), (0, 0, 0, 1), (0, 0, 1, 1)])
+        np.testing.assert_array_equal(svv.to_u32(outs[0]), want[0])
+        np.testing.assert_array_equal(svv.to_u32(outs[2]), want[0][1:])
