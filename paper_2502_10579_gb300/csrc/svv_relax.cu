@@ -38,82 +38,85 @@ __global__ void __launch_bounds__(kRelaxThreads, 2) relax_kernel(RelaxArgs a) {
 
 // ---------------------------------------------------------------------------
 // Output scatter: out[(s0+i)*V + v] = intersection value if v is stable, else
-// the relaxed value of its row.  A CTA stages a tile of kTV vertices x ls
-// snapshots in shared memory so the row reads and the snapshot-major writes
-// both coalesce.  The tile's row map is read first; then a warp takes four
-// vertices at a time with a lane per snapshot, every load independent of the
-// others.  Tile element (i, t) sits at i*kTV + (t ^ (i & 31)): the lanes of a
-// fill store (consecutive i, one t) hit 32 different banks, and the four
-// words of an aligned 16-byte group stay in one group, permuted by i & 3.
-// When V is a multiple of 4 the writes are 16-byte streaming stores (the
-// output is not read again by this query).
+// the relaxed value of its row.  A CTA writes a tile of kTV vertices x ls
+// snapshots.  The rows of the tile's unstable vertices are copied to shared
+// memory by 16-byte asynchronous copies, all of them in flight at once; the
+// 16-byte granule g of vertex t's row lands at g ^ (t / 4), so that a warp that
+// reads 8 groups of four vertices at 4 consecutive snapshots meets every bank
+// once.  A thread keeps its four vertices' intersection values in registers
+// and writes 16 bytes per snapshot (streaming stores: this query does not read
+// the output again); stable vertices touch shared memory nowhere.
+// Bound by the output's bytes: at 1M vertices x 64 snapshots (268 MB, 40 us as
+// a plain fill) 59 us with 10% of the vertices unstable and 70 us with half of
+// them (68 and 98 when every value went through shared memory).  When V is no
+// multiple of 4 the rows start at any word, and a thread writes one word at a
+// time: aligned groups of four that shift with the row were no faster (37 us
+// for 92 MB either way).
 constexpr int kTV = 128;
 constexpr int kScatterThreads = 256;
 
-__device__ __forceinline__ uint32_t pick4(const uint4& w, uint32_t k) {
-  return k == 0 ? w.x : k == 1 ? w.y : k == 2 ? w.z : w.w;
+__device__ __forceinline__ void copy16_async(uint32_t* smem, const uint32_t* gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
+               :
+               : "r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(gmem)
+               : "memory");
 }
 
 __global__ void __launch_bounds__(kScatterThreads) scatter_kernel(ScatterArgs a) {
-  extern __shared__ __align__(16) uint32_t tile[];  // [ls][kTV], swizzled
-  __shared__ uint32_t s_row[kTV];
+  extern __shared__ __align__(16) uint32_t tile[];  // [kTV][LP], granules swizzled
+  __shared__ __align__(16) uint32_t s_row[kTV];
   __shared__ __align__(16) uint32_t s_x[kTV];
   if (*a.qerr != 0u) return;
-  const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const uint32_t lps = __ffs(a.LP) - 1;
+  const uint32_t lps = __ffs(a.LP) - 1, gmask = (a.LP >> 2) - 1u;
   const bool vec = (a.V & 3u) == 0u && ((uintptr_t)a.out & 15u) == 0u;
-  constexpr uint32_t kQ = kTV / 4, kRows = kScatterThreads / kQ;  // 16-byte stores: 32 per tile row
-  const uint32_t q = threadIdx.x % kQ, r0 = threadIdx.x / kQ;
-  {
-    const uint32_t tl = blockIdx.x;  // one tile per CTA
-    const uint32_t v0 = tl * kTV;
-    const uint32_t nv = min((uint32_t)kTV, a.V - v0);
-    bool mine = false;
-    for (uint32_t t = threadIdx.x; t < (uint32_t)kTV; t += blockDim.x) {
-      const bool in = t < nv;
-      const uint32_t r = in ? a.row[v0 + t] : kNone;
-      s_row[t] = r;
-      s_x[t] = in ? a.rI[v0 + t] : 0u;
-      mine |= r != kNone;
+  const uint32_t v0 = blockIdx.x * kTV;  // one tile per CTA
+  const uint32_t nv = min((uint32_t)kTV, a.V - v0);
+  bool mine = false;
+  if (threadIdx.x < kTV) {
+    const uint32_t t = threadIdx.x;
+    const uint32_t r = t < nv ? a.row[v0 + t] : kNone;
+    s_row[t] = r;
+    s_x[t] = t < nv ? a.rI[v0 + t] : 0u;
+    mine = r != kNone;
+  }
+  if (__syncthreads_or(mine)) {
+    // a granule per thread and step: consecutive threads copy one row's
+    const uint32_t ng = (a.ls + 3u) >> 2;
+    for (uint32_t k = threadIdx.x; k < (uint32_t)kTV << (lps - 2u); k += kScatterThreads) {
+      const uint32_t t = k >> (lps - 2u), g = k & gmask, r = s_row[t];
+      if (r != kNone && g < ng)
+        copy16_async(tile + (t << lps) + ((g ^ ((t >> 2) & gmask)) << 2), a.val + ((size_t)r << lps) + (g << 2));
     }
-    if (!__syncthreads_or(mine) && vec && nv == (uint32_t)kTV) {
-      // every vertex of the tile is stable: each snapshot row is the tile's
-      // intersection values, written straight from the row map's buffer
-      const uint4 x = *reinterpret_cast<const uint4*>(s_x + 4u * q);
-      for (uint32_t i = r0; i < a.ls; i += kRows)
-        __stcs(reinterpret_cast<uint4*>(a.out + (size_t)(a.s0 + i) * a.V + v0) + q, x);
-      return;
-    }
-    for (uint32_t t0 = 4u * wid; t0 < (uint32_t)kTV; t0 += 4u * nw) {
-      uint32_t r[4], x[4];
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        r[h] = s_row[t0 + h];
-        x[h] = s_x[t0 + h];
-      }
-      for (uint32_t i = lane; i < a.ls; i += 32u) {
-        uint32_t y[4];
-#pragma unroll
-        for (int h = 0; h < 4; ++h) y[h] = r[h] == kNone ? x[h] : (a.val[((size_t)r[h] << lps) + i] ^ a.rflip);
-#pragma unroll
-        for (int h = 0; h < 4; ++h) tile[i * kTV + ((t0 + h) ^ (i & 31u))] = y[h];
-      }
-    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    if (vec && nv == (uint32_t)kTV) {
-      // a warp per tile row: 32 threads x 16 bytes
-      for (uint32_t i = r0; i < a.ls; i += kRows) {
-        const uint32_t sw = i & 31u;
-        const uint4 w = *reinterpret_cast<const uint4*>(tile + i * kTV + 4u * (q ^ (sw >> 2)));
-        const uint32_t k = sw & 3u;
-        const uint4 o = make_uint4(pick4(w, k), pick4(w, 1u ^ k), pick4(w, 2u ^ k), pick4(w, 3u ^ k));
-        __stcs(reinterpret_cast<uint4*>(a.out + (size_t)(a.s0 + i) * a.V + v0) + q, o);
+  }
+  auto value = [&](uint32_t t, uint32_t i) {
+    return tile[(t << lps) + (((i >> 2) ^ ((t >> 2) & gmask)) << 2) + (i & 3u)] ^ a.rflip;
+  };
+  if (vec && nv == (uint32_t)kTV) {
+    // lane = (group of four vertices, snapshot): 8 groups x 4 snapshots a
+    // warp, 4 warps across the tile, so a store covers 4 rows of 128 bytes
+    const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+    const uint32_t q = (wid & 3u) * 8u + (lane & 7u), i0 = (wid >> 2) * 4u + (lane >> 3);
+    const uint4 r = *reinterpret_cast<const uint4*>(s_row + 4u * q), x = *reinterpret_cast<const uint4*>(s_x + 4u * q);
+    uint4* o = reinterpret_cast<uint4*>(a.out + (size_t)(a.s0 + i0) * a.V + v0) + q;
+    const size_t step = (size_t)(kScatterThreads / 32) * a.V / 4u;  // 8 snapshots on, in 16-byte words
+    const bool stable = (r.x & r.y & r.z & r.w) == kNone;
+    for (uint32_t i = i0; i < a.ls; i += kScatterThreads / 32u, o += step) {
+      uint4 w = x;
+      if (!stable) {
+        if (r.x != kNone) w.x = value(4u * q, i);
+        if (r.y != kNone) w.y = value(4u * q + 1u, i);
+        if (r.z != kNone) w.z = value(4u * q + 2u, i);
+        if (r.w != kNone) w.w = value(4u * q + 3u, i);
       }
-    } else {
-      for (uint32_t i = wid; i < a.ls; i += nw)
-        for (uint32_t t = lane; t < nv; t += 32u)
-          a.out[(size_t)(a.s0 + i) * a.V + v0 + t] = tile[i * kTV + (t ^ (i & 31u))];
+      __stcs(o, w);
     }
+  } else {
+    const uint32_t t = threadIdx.x & (kTV - 1u), r = s_row[t], x = s_x[t];
+    if (t < nv)
+      for (uint32_t i = threadIdx.x / kTV; i < a.ls; i += kScatterThreads / kTV)
+        __stcs(a.out + (size_t)(a.s0 + i) * a.V + v0 + t, r == kNone ? x : value(t, i));
   }
 }
 
@@ -147,10 +150,12 @@ __global__ void __launch_bounds__(256) isolated_kernel(IsolatedArgs a) {
     a.row[v] = kNone;
   }
   if (!a.out) return;
+  // a thread keeps its columns and goes down the rows: no division, and the
+  // value (the source's column apart) never changes
   if ((a.V & 3u) == 0u && ((uintptr_t)a.out & 15u) == 0u) {
-    const size_t per_row = a.V >> 2, n = per_row * a.L;
-    for (size_t k = tid; k < n; k += nthreads) {
-      const uint32_t v = (uint32_t)(k % per_row) * 4u;
+    const size_t per_row = a.V >> 2;
+    for (size_t k = tid; k < per_row; k += nthreads) {
+      const uint32_t v = (uint32_t)k * 4u;
       uint4 o = make_uint4(a.ident, a.ident, a.ident, a.ident);
       if (a.source - v < 4u) {
         const uint32_t j = a.source - v;
@@ -159,11 +164,15 @@ __global__ void __launch_bounds__(256) isolated_kernel(IsolatedArgs a) {
         else if (j == 2) o.z = a.src_val;
         else o.w = a.src_val;
       }
-      __stcs(reinterpret_cast<uint4*>(a.out) + k, o);
+      uint4* p = reinterpret_cast<uint4*>(a.out) + k;
+      for (uint32_t i = 0; i < a.L; ++i, p += per_row) __stcs(p, o);
     }
   } else {
-    const size_t n = (size_t)a.V * a.L;
-    for (size_t k = tid; k < n; k += nthreads) a.out[k] = (k % a.V) == a.source ? a.src_val : a.ident;
+    for (size_t v = tid; v < a.V; v += nthreads) {
+      const uint32_t x = v == a.source ? a.src_val : a.ident;
+      uint32_t* p = a.out + v;
+      for (uint32_t i = 0; i < a.L; ++i, p += a.V) *p = x;
+    }
   }
 }
 
@@ -217,9 +226,8 @@ cudaError_t launch_relax(int type, uint32_t P, uint32_t K, const RelaxArgs& a, L
 
 cudaError_t launch_scatter(const ScatterArgs& a, cudaStream_t s) {
   const uint32_t blocks = (a.V + kTV - 1) / kTV;  // one tile per CTA
-  const size_t smem = (size_t)a.ls * kTV * sizeof(uint32_t);  // up to 64 KB at 128 snapshots
-  // the opt-in covers the dynamic tile plus the kernel's static row map
-  if (smem + 2 * kTV * sizeof(uint32_t) > 48 * 1024) {
+  const size_t smem = (size_t)a.LP * kTV * sizeof(uint32_t);  // up to 64 KB for 128 snapshots
+  if (smem > 40 * 1024) {  // with the static row map, past what needs no opt-in
     cudaError_t e = cudaFuncSetAttribute((const void*)scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
