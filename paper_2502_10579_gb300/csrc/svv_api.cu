@@ -498,10 +498,10 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
   const uint64_t nblk = (uint64_t)c->num_sms * 4;
   if ((st = alloc_n(c, c->scratch_bufs, V, &c->rI)) || (st = alloc_n(c, c->scratch_bufs, V, &c->rU)) ||
       (st = alloc_n(c, c->scratch_bufs, V, &c->stamp)) || (st = alloc_n(c, c->scratch_bufs, V, &c->row)) ||
-      (st = alloc_n(c, c->scratch_bufs, V, &c->uv)) || (st = alloc_n(c, c->scratch_bufs, 4 * nblk, &c->part)) ||
-      (st = alloc_n(c, c->scratch_bufs, 2ull * V, &c->qcnt)) || (st = alloc_n(c, c->scratch_bufs, 2ull * V, &c->cur)) ||
+      (st = alloc_n(c, c->scratch_bufs, V, &c->uv)) || (st = alloc_n(c, c->scratch_bufs, 8 * nblk, &c->part)) ||
       (st = alloc_n(c, c->scratch_bufs, V, &c->qrow)) ||
       (st = alloc_n(c, c->scratch_bufs, std::max<uint32_t>(E2, 1), &c->qcw)) ||
+      (st = alloc_n(c, c->scratch_bufs, std::max<uint32_t>(NF, 1), &c->qmcw)) ||
       (st = alloc_n(c, c->scratch_bufs, qcap, &c->q0)) || (st = alloc_n(c, c->scratch_bufs, qcap, &c->q1)) ||
       (st = alloc_n(c, c->scratch_bufs, ucap, &c->units)) ||
       (st = alloc_n(c, c->scratch_bufs, kNumCtl, &c->ctl)) || (st = alloc_n(c, c->scratch_bufs, 1, &c->qerr)) ||
@@ -647,10 +647,9 @@ svv_status enqueue_tail(svv_ctx* c, int t, uint32_t wb, uint32_t wl, uint32_t* o
   q.units = c->units;
   q.ucap = c->ucap;
   q.cshift = c->qrs_cs;
-  q.qcnt = c->qcnt;
   q.qrow = c->qrow;
-  q.cur = c->cur;
   q.qcw = c->qcw;
+  q.qmcw = c->qmcw;
   q.qmask = c->qmask;
   q.ecap = c->ecap;
   q.mcap = c->mcap;
@@ -685,6 +684,7 @@ svv_status enqueue_tail(svv_ctx* c, int t, uint32_t wb, uint32_t wl, uint32_t* o
     r.uv = c->uv;
     r.qrow = c->qrow;
     r.qcw = c->qcw;
+    r.qmcw = c->qmcw;
     r.qmask = c->qmask;
     r.counts = &(c->ctl + 2)->aux[0];
     r.val = c->val;

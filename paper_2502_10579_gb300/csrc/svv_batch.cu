@@ -124,10 +124,9 @@ __device__ bool run_instance(const BatchArgs& b, const BatchInstance& q, uint32_
   r.units = sc.units;
   r.ucap = sc.ucap;
   r.cshift = b.qrs_cs;
-  r.qcnt = sc.qcnt;
   r.qrow = sc.qrow;
-  r.cur = sc.cur;
   r.qcw = sc.qcw;
+  r.qmcw = sc.qmcw;
   r.qmask = sc.qmask;
   r.ecap = sc.ecap;
   r.mcap = sc.mcap;
@@ -161,6 +160,7 @@ __device__ bool run_instance(const BatchArgs& b, const BatchInstance& q, uint32_
     x.uv = sc.uv;
     x.qrow = sc.qrow;
     x.qcw = sc.qcw;
+    x.qmcw = sc.qmcw;
     x.qmask = sc.qmask;
     x.counts = &(tc + 3)->aux[0];
     x.val = sc.val;

@@ -170,9 +170,9 @@ struct svv_ctx {
   // query scratch (sized at load from V and E; the L-dependent part on demand)
   std::vector<void*> scratch_bufs;
   uint32_t *rI = nullptr, *rU = nullptr, *stamp = nullptr, *row = nullptr, *uv = nullptr;
-  uint32_t *part = nullptr, *qcnt = nullptr, *cur = nullptr, *qerr = nullptr;
+  uint32_t *part = nullptr, *qerr = nullptr;
   uint4* qrow = nullptr;
-  uint2* qcw = nullptr;
+  uint2 *qcw = nullptr, *qmcw = nullptr;
   unsigned long long *q0 = nullptr, *q1 = nullptr, *units = nullptr;
   uint32_t qcap = 0, ucap = 0, ecap = 0;
   svv::TeamCtl* ctl = nullptr;
@@ -188,9 +188,9 @@ struct svv_ctx {
   // a two-query group's tails in one relaxation launch: both queries' rows,
   // subgraph edges and masks in one set of arrays (allocated on first use)
   std::vector<void*> pair_bufs;
-  uint32_t *p_uv = nullptr, *p_qcnt = nullptr, *p_cur = nullptr, *p_stamp = nullptr, *p_row1 = nullptr;
+  uint32_t *p_uv = nullptr, *p_stamp = nullptr, *p_row1 = nullptr;
   uint4* p_qrow = nullptr;
-  uint2* p_qcw = nullptr;
+  uint2 *p_qcw = nullptr, *p_qmcw = nullptr;
   uint64_t* p_qmask = nullptr;
   uint32_t* p_val = nullptr;
   unsigned long long *p_q0 = nullptr, *p_q1 = nullptr, *p_units = nullptr;

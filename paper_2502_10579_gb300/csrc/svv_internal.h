@@ -129,22 +129,21 @@ struct QrsArgs {
   const uint32_t* rU;     // union-graph values
   uint32_t* row;          // [V] vertex -> row, kNone if stable
   uint32_t* uv;           // [V] row -> vertex
-  uint32_t* part;         // [4 * gridDim] per-CTA partial sums
+  uint32_t* part;         // [8 * gridDim] per-CTA sums
   unsigned long long* units;  // row | chunk << 32 over unstable rows
   uint32_t ucap;
   uint32_t cshift;
-  uint32_t* qcnt;         // [2V] per row: (#all-window edges, #other edges)
-  uint4* qrow;            // [V] per row: {start, all-window end, mask base, end}
-  uint32_t* cur;          // [2V] fill cursors
-  uint2* qcw;             // [E] (target row, weight)
-  uint64_t* qmask;        // [NF*QW] window-rebased masks
+  uint4* qrow;            // [V] per row: {first all-window edge, first other edge, how many of each}
+  uint2* qcw;             // [E] all-window edges (target row, weight): room for all out-edges of every row
+  uint2* qmcw;            // [NF] the others
+  uint64_t* qmask;        // [NF*QW] their window-rebased masks
   uint32_t ecap;
   unsigned long long mcap;  // words
   TeamCtl* ctl;           // aux[0]=U, aux[1]=#units, aux[2]=E_Q, aux[3]=#masked
   uint32_t* qerr;
   unsigned long long spin_ns;
   unsigned long long* trace;  // optional: start ns of each of the five passes, then the end
-  uint32_t rowcap;        // rows the row arrays hold (uv, qrow; qcnt and cur hold 2 per row)
+  uint32_t rowcap;        // rows the row arrays hold (uv, qrow)
   // a second query extracted in the same launch (rI1 null: none), same window
   // length: its rows, units, edges and masks follow the first query's; its
   // number of rows goes to counts1_out[0] (aux[0] holds the first query's)
@@ -165,6 +164,7 @@ struct RelaxArgs {
   const uint32_t* uv;
   const uint4* qrow;
   const uint2* qcw;
+  const uint2* qmcw;
   const uint64_t* qmask;
   const unsigned int* counts;  // qrs team aux: [0]=U
   // a second query relaxed in the same launch (counts1 null: none): its rows
@@ -242,9 +242,9 @@ struct BatchInstance {
 
 // per-team query scratch (same roles as the single-query scratch)
 struct TeamScratch {
-  uint32_t *rI, *rU, *stamp, *row, *uv, *part, *qcnt, *cur;
+  uint32_t *rI, *rU, *stamp, *row, *uv, *part;
   uint4* qrow;
-  uint2* qcw;
+  uint2 *qcw, *qmcw;
   uint64_t* qmask;
   uint32_t* val;
   unsigned long long *q0, *q1, *units;

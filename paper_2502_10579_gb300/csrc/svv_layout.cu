@@ -334,9 +334,10 @@ __global__ void __launch_bounds__(256) rowd_kernel(const uint32_t* rp, const uin
 // row descriptors from the row offsets and the (host) prefix counts of partial edges
 svv_status build_rowd(svv_ctx* c, const uint32_t* nfp, uint4* rowd) {
   const uint32_t V = c->g.V;
-  cudaError_t e = cudaMemcpy(c->cur, nfp, ((size_t)V + 1) * 4, cudaMemcpyHostToDevice);  // cur holds 2V words
+  uint32_t* tmp = reinterpret_cast<uint32_t*>(c->q0);  // more than 2V words
+  cudaError_t e = cudaMemcpy(tmp, nfp, ((size_t)V + 1) * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) {
-    rowd_kernel<<<blocks_for(V, 1024), 256>>>(c->g.rp, c->cur, V, rowd);
+    rowd_kernel<<<blocks_for(V, 1024), 256>>>(c->g.rp, tmp, V, rowd);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(0);
@@ -351,10 +352,11 @@ svv_status build_pull(svv_ctx* c) {
   const DevGraph& g = c->g;
   const uint32_t V = g.V;
   cudaError_t e = cudaSuccess;
-  uint32_t *deg = c->stamp, *deg_p = c->rI, *start = c->rU, *width = c->row, *sbase = c->uv, *sitem = c->cur;
-  uint2* tpos = reinterpret_cast<uint2*>(c->qcnt);
+  uint32_t *deg = c->stamp, *deg_p = c->rI, *start = c->rU, *width = c->row, *sbase = c->uv;
+  uint32_t* sitem = reinterpret_cast<uint32_t*>(c->q0);
+  uint2* tpos = reinterpret_cast<uint2*>(c->qrow);
   unsigned long long* meta = reinterpret_cast<unsigned long long*>(c->part);
-  uint32_t *hist = c->part + 2 * kMeta, *off = hist + kBins;  // part holds 16 words per SM
+  uint32_t *hist = c->part + 2 * kMeta, *off = hist + kBins;  // part holds 32 words per SM
   uint32_t* segoff = off + kBins;
   uint32_t* counts = reinterpret_cast<uint32_t*>(c->ctl);  // cleared by every query
   static_assert(sizeof(TeamCtl) * kNumCtl >= 256 * kSortBlocks * sizeof(uint32_t), "sort counters");

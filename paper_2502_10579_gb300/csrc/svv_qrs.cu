@@ -14,19 +14,24 @@
 // come first (Section 4.1), followed by the rest with masks rebased so that bit
 // i is snapshot win_begin+i.
 //
-// One cooperative launch, five phases separated by the team barrier:
-//   P1 per-CTA counts of unstable vertices and their work units;
-//   P2 rows in vertex order (CTA offsets from P1), row -> vertex map, units;
-//   P3 per-row edge counts (all-window / masked);
-//   P4 exclusive scan of the row counts -> row descriptors and fill cursors;
-//   P5 fill.
+// One cooperative launch, three phases separated by the team barrier:
+//   P1 per-CTA counts of unstable vertices, their work units and out-edges;
+//   P2 rows in vertex order (CTA offsets from P1), row -> vertex map, units,
+//      and each row's place in the edge arrays, with room for all its out-edges;
+//   P3 fill: the kept edges of every unit behind those its row already holds.
+// The edges are walked once.  Counting the kept edges first, to pack the rows,
+// walked them twice, at one CTA per SM (114 registers): 121 us instead of 79 at
+// scale 20 with 111K unstable vertices, 458 instead of 311 with 533K.  Two CTAs
+// per SM at 64 registers; three (40, with spills) took 85 and 353 us.  Bound by
+// the walk's chain of dependent loads (unit, row, target, row map) and its
+// returning atomics.
 #include "svv_qrs.cuh"
 
 namespace svv {
 
 constexpr int kQrsThreads = 512;
 
-__global__ void __launch_bounds__(kQrsThreads) qrs_kernel(QrsArgs a) {
+__global__ void __launch_bounds__(kQrsThreads, 2) qrs_kernel(QrsArgs a) {
   __shared__ TeamBar s_bar;
   const Team t{a.ctl, a.qerr, gridDim.x, blockIdx.x, a.spin_ns, &s_bar};
   t.begin();

@@ -9,77 +9,77 @@ namespace svv {
 
 
 
-// exclusive block scan of two counters; block totals in ta/tb
-__device__ __forceinline__ void block_excl_scan2(uint32_t a, uint32_t b, uint32_t& ea, uint32_t& eb,
-                                                 uint32_t& ta, uint32_t& tb) {
-  __shared__ uint32_t s_a[33], s_b[33];
-  const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const uint32_t ia = warp_incl_scan(a, lane), ib = warp_incl_scan(b, lane);
-  if (lane == 31) {
-    s_a[wid] = ia;
-    s_b[wid] = ib;
+// what a range of vertices needs in the subgraph's arrays
+struct QrsSum {
+  uint32_t rows, units, deg, part;  // unstable vertices, their units, out-edges and partial out-edges
+  __device__ __forceinline__ void add(const QrsSum& o) {
+    rows += o.rows;
+    units += o.units;
+    deg += o.deg;
+    part += o.part;
   }
-  __syncthreads();
-  if (wid == 0) {
-    const uint32_t xa = lane < nw ? s_a[lane] : 0u, xb = lane < nw ? s_b[lane] : 0u;
-    const uint32_t ya = warp_incl_scan(xa, lane), yb = warp_incl_scan(xb, lane);
-    if (lane < nw) {
-      s_a[lane] = ya - xa;
-      s_b[lane] = yb - xb;
-    }
-    if (lane == 31) {
-      s_a[32] = ya;
-      s_b[32] = yb;
-    }
-  }
-  __syncthreads();
-  ea = s_a[wid] + ia - a;
-  eb = s_b[wid] + ib - b;
-  ta = s_a[32];
-  tb = s_b[32];
-  __syncthreads();
+};
+
+__device__ __forceinline__ QrsSum warp_incl_scan(QrsSum x, unsigned lane) {
+  return QrsSum{warp_incl_scan(x.rows, lane), warp_incl_scan(x.units, lane), warp_incl_scan(x.deg, lane),
+                warp_incl_scan(x.part, lane)};
 }
 
-// sum of four counters over the block
-__device__ __forceinline__ void block_sum4(uint32_t& a, uint32_t& b, uint32_t& c, uint32_t& d) {
-  __shared__ uint32_t s[4][32];
+// sums over the warps before this one, and over the block
+__device__ __forceinline__ void block_sums(const QrsSum& warp_total, QrsSum& before, QrsSum& total) {
+  __shared__ QrsSum s[32];
   const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(kFullMask, a, o);
-    b += __shfl_xor_sync(kFullMask, b, o);
-    c += __shfl_xor_sync(kFullMask, c, o);
-    d += __shfl_xor_sync(kFullMask, d, o);
-  }
-  if (lane == 0) {
-    s[0][wid] = a;
-    s[1][wid] = b;
-    s[2][wid] = c;
-    s[3][wid] = d;
-  }
+  if (lane == 0) s[wid] = warp_total;
   __syncthreads();
-  a = b = c = d = 0u;
+  before = total = QrsSum{};
   for (unsigned i = 0; i < nw; ++i) {
-    a += s[0][i];
-    b += s[1][i];
-    c += s[2][i];
-    d += s[3][i];
+    if (i < wid) before.add(s[i]);
+    total.add(s[i]);
   }
   __syncthreads();
 }
 
-// Walk the edges of every unit in the queue (warp-balanced, as in the solve)
-// and classify each edge: all-window (F) or masked (M) kept edge.
-// FILL=false: add per-row counts; FILL=true: write the edges.
-// With a second query (a.rI1), rows from U0 on are that query's: its edges
-// are classified against its own row map and window.
-template <bool FILL>
-__device__ void qrs_walk(const QrsArgs& a, const Team& t, uint32_t NU, uint32_t U0, unsigned* ticket) {
+__device__ __forceinline__ QrsSum warp_sum(const QrsSum& x) {
+  return QrsSum{__reduce_add_sync(kFullMask, x.rows), __reduce_add_sync(kFullMask, x.units),
+                __reduce_add_sync(kFullMask, x.deg), __reduce_add_sync(kFullMask, x.part)};
+}
+
+// a vertex's share, if its bounds differ (with pruning off every vertex has a row)
+__device__ __forceinline__ QrsSum vertex_share(const QrsArgs& a, uint32_t v, bool unstable) {
+  if (!unstable) return QrsSum{};
+  const uint4 rd = __ldg(a.g.rowd + v);
+  const uint32_t deg = rd.y - rd.x;
+  return QrsSum{1u, (deg + (1u << a.cshift) - 1u) >> a.cshift, deg, rd.y - rd.z};
+}
+
+// bit h of the result: vertex v + h (< hi) is unstable; v is a multiple of 4
+__device__ __forceinline__ uint32_t unstable4(const QrsArgs& a, const uint32_t* I, const uint32_t* U, uint32_t v,
+                                              uint32_t hi) {
+  if (v >= hi) return 0u;
+  const uint32_t in = hi - v < 4u ? (1u << (hi - v)) - 1u : 15u;
+  if (!a.prune) return in;
+  if (in == 15u) {
+    const uint4 x = *reinterpret_cast<const uint4*>(I + v), y = *reinterpret_cast<const uint4*>(U + v);
+    return (x.x != y.x ? 1u : 0u) | (x.y != y.y ? 2u : 0u) | (x.z != y.z ? 4u : 0u) | (x.w != y.w ? 8u : 0u);
+  }
+  uint32_t m = 0;
+  for (uint32_t h = 0; h < hi - v; ++h) m |= (I[v + h] != U[v + h] ? 1u : 0u) << h;
+  return m;
+}
+
+// Walk the edges of every unit in the queue (warp-balanced, as in the solve),
+// classify each edge as all-window (F) or masked (M) kept edge, and write the
+// kept ones behind those their rows already hold.  Returns (in lane 0) the
+// numbers of kept and of masked edges.  With a second query (a.rI1), rows from
+// U0 on are that query's: its edges are classified against its own row map and
+// window.
+__device__ __forceinline__ uint2 qrs_fill(const QrsArgs& a, const Team& t, uint32_t NU, uint32_t U0, unsigned* ticket) {
+  uint2 kept = make_uint2(0u, 0u);
   const DevGraph& g = a.g;
   const unsigned lane = threadIdx.x & 31u;
   const unsigned lt = (1u << lane) - 1u;
   const uint32_t nwarps = t.nthreads() >> 5;
-  const uint32_t gwarp = t.tid() >> 5;
+  const uint32_t gwarp = (threadIdx.x >> 5) * t.nblocks + t.rank;
   const Batches bt{NU, batch_size(NU, nwarps, 32u), nwarps, gwarp, ticket};
   const uint32_t tk = bt.tk;
   for (uint32_t t0 = bt.first(); t0 < NU; t0 = bt.next(lane)) {
@@ -106,7 +106,7 @@ __device__ void qrs_walk(const QrsArgs& a, const Team& t, uint32_t NU, uint32_t 
       int kk[2];
       uint32_t rkk[2], rx[2], w[2];
       bool isF[2], isM[2];
-      const uint64_t* m[2];
+      uint32_t mi[2];  // a partial edge's index in the partial list
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const uint32_t p = p0 + 32u * h + lane;
@@ -121,7 +121,7 @@ __device__ void qrs_walk(const QrsArgs& a, const Team& t, uint32_t NU, uint32_t 
         isF[h] = isM[h] = false;
         rx[h] = kNone;
         w[h] = 0;
-        m[h] = nullptr;
+        mi[h] = 0u;
         if (p < total) {
           const uint32_t e = bk + (p - (ik - ck));
           const uint2 ew = __ldg(g.cw + e);
@@ -132,9 +132,9 @@ __device__ void qrs_walk(const QrsArgs& a, const Team& t, uint32_t NU, uint32_t 
             if (e < fk) {
               isF[h] = true;
             } else {
-              m[h] = g.nfmask + (size_t)(nk + (e - fk)) * g.W;
+              mi[h] = nk + (e - fk);
               bool any, all;
-              window_any_all(m[h], q1 ? a.win1 : a.win, any, all);
+              window_any_all(g.nfmask + (size_t)mi[h] * g.W, q1 ? a.win1 : a.win, any, all);
               isF[h] = all;
               isM[h] = any && !all;
             }
@@ -149,39 +149,36 @@ __device__ void qrs_walk(const QrsArgs& a, const Team& t, uint32_t NU, uint32_t 
         const unsigned bF = __ballot_sync(kFullMask, isF[h]), bM = __ballot_sync(kFullMask, isM[h]);
         const int leader = __ffs(grp) - 1;
         const uint32_t nF = __popc(grp & bF), nM = __popc(grp & bM);
-        if (!FILL) {
-          if (lane == (unsigned)leader && p < total) {
-            if (nF) atomicAdd(a.qcnt + 2u * rk, nF);
-            if (nM) atomicAdd(a.qcnt + 2u * rk + 1u, nM);
-          }
-        } else {
-          uint32_t baseF = 0, baseM = 0;
-          if (lane == (unsigned)leader && p < total) {
-            if (nF) baseF = atomicAdd(a.cur + 2u * rk, nF);
-            if (nM) baseM = atomicAdd(a.cur + 2u * rk + 1u, nM);
-          }
-          baseF = __shfl_sync(kFullMask, baseF, leader);
-          baseM = __shfl_sync(kFullMask, baseM, leader);
-          if (isF[h]) {
-            const uint32_t pos = baseF + __popc(grp & bF & lt);
-            a.qcw[pos] = make_uint2(rx[h], w[h]);
-          } else if (isM[h]) {
-            const uint32_t pos = baseM + __popc(grp & bM & lt);
-            a.qcw[pos] = make_uint2(rx[h], w[h]);
-            const uint4 d = __ldcg(a.qrow + rk);
-            uint64_t* out = a.qmask + (size_t)(d.z + (pos - d.y)) * a.QW;
-            const uint32_t wb = (a.rI1 && rk >= U0) ? a.win1.b : a.win.b;
-            for (uint32_t j = 0; j < a.QW; ++j) {
-              uint64_t word = mask_extract(m[h], g.W, wb + 64u * j);
-              const uint32_t left = a.win.l - 64u * j;
-              if (left < 64u) word &= (1ull << left) - 1ull;
-              out[j] = word;
-            }
+        uint32_t baseF = 0, baseM = 0;
+        uint4* d = a.qrow + rk;
+        uint2 at = make_uint2(0u, 0u);
+        if (lane == (unsigned)leader && p < total && (nF || nM)) {
+          at = __ldcg(reinterpret_cast<const uint2*>(d));  // {first full edge, first masked edge}
+          if (nF) baseF = atomicAdd(&d->z, nF);
+          if (nM) baseM = atomicAdd(&d->w, nM);
+        }
+        baseF = __shfl_sync(kFullMask, at.x + baseF, leader);
+        baseM = __shfl_sync(kFullMask, at.y + baseM, leader);
+        if (isF[h]) {
+          a.qcw[baseF + __popc(grp & bF & lt)] = make_uint2(rx[h], w[h]);
+        } else if (isM[h]) {
+          const uint32_t pos = baseM + __popc(grp & bM & lt);
+          a.qmcw[pos] = make_uint2(rx[h], w[h]);
+          uint64_t* out = a.qmask + (size_t)pos * a.QW;
+          const uint32_t wb = (a.rI1 && rk >= U0) ? a.win1.b : a.win.b;
+          for (uint32_t j = 0; j < a.QW; ++j) {
+            uint64_t word = mask_extract(g.nfmask + (size_t)mi[h] * g.W, g.W, wb + 64u * j);
+            const uint32_t left = a.win.l - 64u * j;
+            if (left < 64u) word &= (1ull << left) - 1ull;
+            out[j] = word;
           }
         }
+        kept.x += __popc(bF) + __popc(bM);
+        kept.y += __popc(bM);
       }
     }
   }
+  return kept;
 }
 
 __device__ inline bool qrs_team(const QrsArgs& a, const Team& t) {
@@ -190,180 +187,123 @@ __device__ inline bool qrs_team(const QrsArgs& a, const Team& t) {
   const unsigned nb = t.nblocks, b = t.rank, tid = threadIdx.x;
   if (cta_read(a.qerr) != 0u) return false;
   const uint32_t V = g.V;
-  const uint32_t C = 1u << a.cshift;
-  // A second query (a.rI1) is extracted in the same launch: its rows follow
-  // the first query's, its units follow theirs, and the row scan and the
-  // fill run over both ranges at once.
+  // A second query (a.rI1) is extracted in the same launch: its rows, units
+  // and edges follow the first query's.
   const int nq = a.rI1 ? 2 : 1;
 
-  // ---- P1: unstable vertices and their units, per CTA vertex range and query
+  // ---- P1: what each CTA's vertex range needs, per query
   if (a.trace && b == 0 && tid == 0) a.trace[0] = global_ns();
   const unsigned long long per = (((unsigned long long)V + nb - 1) / nb + 31ull) & ~31ull;
   const uint32_t lo = (uint32_t)min((unsigned long long)V, per * b);
   const uint32_t hi = (uint32_t)min((unsigned long long)V, per * b + per);
-  {
-    uint32_t cnt = 0, nun = 0, cnt1 = 0, nun1 = 0;
-    for (uint32_t v = lo + tid; v < hi; v += blockDim.x) {
-      const uint32_t nv = (__ldg(g.rp + v + 1) - __ldg(g.rp + v) + C - 1u) >> a.cshift;
-      if (!a.prune || a.rI[v] != a.rU[v]) {
-        ++cnt;
-        nun += nv;
-      }
-      if (nq > 1 && (!a.prune || a.rI1[v] != a.rU1[v])) {
-        ++cnt1;
-        nun1 += nv;
-      }
+  for (int qi = 0; qi < nq; ++qi) {
+    const uint32_t* qI = qi ? a.rI1 : a.rI;
+    const uint32_t* qU = qi ? a.rU1 : a.rU;
+    QrsSum sum{};
+    for (uint32_t v = lo + 4u * tid; v < hi; v += 4u * blockDim.x) {
+      uint32_t m = unstable4(a, qI, qU, v, hi);
+      for (; m; m &= m - 1u) sum.add(vertex_share(a, v + __ffs(m) - 1, true));
     }
-    block_sum4(cnt, nun, cnt1, nun1);
-    if (tid == 0) {
-      a.part[4 * b] = cnt;
-      a.part[4 * b + 1] = nun;
-      a.part[4 * b + 2] = cnt1;
-      a.part[4 * b + 3] = nun1;
-    }
+    QrsSum before, total;
+    block_sums(warp_sum(sum), before, total);
+    if (tid == 0) reinterpret_cast<uint4*>(a.part)[2 * b + qi] = make_uint4(total.rows, total.units, total.deg, total.part);
   }
   if (!t.sync()) return false;
 
-  // ---- P2: rows and units in vertex order, the first query's then the second's
+  // ---- P2: rows and units in vertex order, the first query's then the
+  // second's; a row has room for all its out-edges, so nothing is counted first
   if (a.trace && b == 0 && tid == 0) a.trace[1] = global_ns();
-  uint32_t U = 0, NU = 0, U0 = 0;
+  QrsSum base{};  // the queries before
+  uint32_t U0 = 0;
   for (int qi = 0; qi < nq; ++qi) {
     const uint32_t* qI = qi ? a.rI1 : a.rI;
     const uint32_t* qU = qi ? a.rU1 : a.rU;
     uint32_t* qrowmap = qi ? a.row1 : a.row;
-    uint32_t o_r = 0, o_u = 0, t_r = 0, t_u = 0;
+    QrsSum mine{}, all{};
     for (uint32_t j = tid; j < nb; j += blockDim.x) {
-      const uint32_t pr = ld_cg(a.part + 4 * j + 2 * qi), pu = ld_cg(a.part + 4 * j + 2 * qi + 1);
-      t_r += pr;
-      t_u += pu;
-      if (j < b) {
-        o_r += pr;
-        o_u += pu;
-      }
+      const uint4 x = __ldcg(reinterpret_cast<const uint4*>(a.part) + 2 * j + qi);
+      const QrsSum s{x.x, x.y, x.z, x.w};
+      all.add(s);
+      if (j < b) mine.add(s);
     }
-    block_sum4(o_r, o_u, t_r, t_u);
-    const uint32_t rbase = U, ubase = NU;  // after the first query's rows and units
-    U += t_r;
-    NU += t_u;
-    if (qi == 0) U0 = t_r;
+    QrsSum none, at, total;
+    block_sums(warp_sum(mine), none, at);
+    block_sums(warp_sum(all), none, total);
+    at.add(base);  // where this CTA's range begins
+    base.add(total);
+    if (qi == 0) U0 = total.rows;
     if (b == 0 && tid == 0) {
       if (qi == 0) {
-        c->aux[0] = t_r;
-        c->aux[1] = t_u;
+        c->aux[0] = total.rows;
+        c->aux[1] = total.units;
       } else {
-        a.counts1_out[0] = t_r;
+        a.counts1_out[0] = total.rows;
       }
     }
-    if (NU > a.ucap || U > a.rowcap) {
+    if (base.units > a.ucap || base.rows > a.rowcap || base.deg > a.ecap ||
+        (unsigned long long)base.part * a.QW > a.mcap) {
       if (tid == 0) set_err(c, a.qerr, kErrInternal);
       return false;  // every CTA sees the same totals and leaves here
     }
-    for (uint32_t base = lo; base < hi; base += blockDim.x) {
-      const uint32_t v = base + tid;
-      uint32_t flag = 0, nu = 0;
-      if (v < hi && (!a.prune || qI[v] != qU[v])) {
-        flag = 1;
-        nu = (__ldg(g.rp + v + 1) - __ldg(g.rp + v) + C - 1u) >> a.cshift;
-      }
-      uint32_t ef, eu, tf, tu;
-      block_excl_scan2(flag, nu, ef, eu, tf, tu);
-      const uint32_t r = rbase + o_r + ef;
-      if (v < hi) {
-        qrowmap[v] = flag ? r : kNone;
-        if (flag) {
-          a.uv[r] = v;
-          a.qcnt[2 * r] = 0u;
-          a.qcnt[2 * r + 1] = 0u;
+    const unsigned lane = tid & 31u;
+    for (uint32_t v0 = lo; v0 < hi; v0 += 4u * blockDim.x) {
+      const uint32_t v = v0 + 4u * tid;
+      const uint32_t m = unstable4(a, qI, qU, v, hi);
+      QrsSum sum{};
+#pragma unroll
+      for (uint32_t h = 0; h < 4u; ++h) sum.add(vertex_share(a, v + h, (m >> h) & 1u));
+      const QrsSum incl = warp_incl_scan(sum, lane);
+      const QrsSum wt{__shfl_sync(kFullMask, incl.rows, 31), __shfl_sync(kFullMask, incl.units, 31),
+                      __shfl_sync(kFullMask, incl.deg, 31), __shfl_sync(kFullMask, incl.part, 31)};
+      QrsSum before, btotal;
+      block_sums(wt, before, btotal);
+      QrsSum p = at;  // of this lane's first vertex
+      p.add(before);
+      p.rows += incl.rows - sum.rows;
+      p.units += incl.units - sum.units;
+      p.deg += incl.deg - sum.deg;
+      p.part += incl.part - sum.part;
+      at.add(btotal);
+#pragma unroll 1
+      for (uint32_t h = 0; h < 4u; ++h) {
+        const bool on = (m >> h) & 1u;
+        const QrsSum own = vertex_share(a, v + h, on);  // again: cheaper than keeping four
+        if (v + h < hi) {
+          qrowmap[v + h] = on ? p.rows : kNone;
+          if (on) {
+            a.uv[p.rows] = v + h;
+            a.qrow[p.rows] = make_uint4(p.deg, p.part, 0u, 0u);
+          }
         }
+        // the warp writes its vertices' units together, so a hub's hundreds
+        // of units do not serialise on one thread
+        const uint32_t nu = own.units;
+        const uint32_t ui = warp_incl_scan(nu, lane);
+        const uint32_t wtot = __shfl_sync(kFullMask, ui, 31);
+        for (uint32_t j0 = 0; j0 < wtot; j0 += 32u) {
+          const uint32_t j = j0 + lane;
+          const int k = warp_owner(ui, j < wtot ? j : wtot - 1u);
+          const uint32_t ik = __shfl_sync(kFullMask, ui, k), nk = __shfl_sync(kFullMask, nu, k);
+          const uint32_t rk = __shfl_sync(kFullMask, p.rows, k), ek = __shfl_sync(kFullMask, p.units, k);
+          const uint32_t jj = j - (ik - nk);
+          if (j < wtot) a.units[ek + jj] = (unsigned long long)rk | ((unsigned long long)jj << 32);
+        }
+        p.add(own);
       }
-      // the warp writes its vertices' units together, so a hub's hundreds
-      // of units do not serialise on one thread
-      const unsigned lane = tid & 31u;
-      const uint32_t incl = warp_incl_scan(nu, lane);
-      const uint32_t wtot = __shfl_sync(kFullMask, incl, 31);
-      for (uint32_t j0 = 0; j0 < wtot; j0 += 32u) {
-        const uint32_t j = j0 + lane;
-        const int k = warp_owner(incl, j < wtot ? j : wtot - 1u);
-        const uint32_t ik = __shfl_sync(kFullMask, incl, k), nk = __shfl_sync(kFullMask, nu, k);
-        const uint32_t rk = __shfl_sync(kFullMask, r, k), ek = __shfl_sync(kFullMask, eu, k);
-        const uint32_t jj = j - (ik - nk);
-        if (j < wtot) a.units[ubase + o_u + ek + jj] = (unsigned long long)rk | ((unsigned long long)jj << 32);
-      }
-      o_r += tf;
-      o_u += tu;
     }
   }
   if (!t.sync()) return false;
 
-  // ---- P3: per-row counts of kept edges
-  if (a.trace && b == 0 && tid == 0) a.trace[2] = global_ns();
-  qrs_walk<false>(a, t, NU, U0, &c->ticket[0]);
-  if (!t.sync()) return false;
-
-  // ---- P4: scan rows
-  if (a.trace && b == 0 && tid == 0) a.trace[3] = global_ns();
-  const unsigned long long rper = (((unsigned long long)U + nb - 1) / nb + 31ull) & ~31ull;
-  const uint32_t rlo = (uint32_t)min((unsigned long long)U, rper * b);
-  const uint32_t rhi = (uint32_t)min((unsigned long long)U, rper * b + rper);
-  {
-    uint32_t se = 0, sm = 0, z0 = 0, z1 = 0;
-    for (uint32_t r = rlo + tid; r < rhi; r += blockDim.x) {
-      const uint32_t f = ld_cg(a.qcnt + 2 * r), m = ld_cg(a.qcnt + 2 * r + 1);
-      se += f + m;
-      sm += m;
-    }
-    block_sum4(se, sm, z0, z1);
-    if (tid == 0) {
-      a.part[2 * nb + 2 * b] = se;
-      a.part[2 * nb + 2 * b + 1] = sm;
-    }
+  // ---- P3: fill
+  if (a.trace && b == 0 && tid == 0) a.trace[2] = a.trace[3] = a.trace[4] = global_ns();
+  const uint2 kept = qrs_fill(a, t, base.units, U0, &c->ticket[0]);
+  QrsSum none, total;
+  block_sums(QrsSum{kept.x, kept.y, 0u, 0u}, none, total);
+  if (tid == 0) {
+    if (total.rows) atomicAdd(&c->aux[2], total.rows);
+    if (total.units) atomicAdd(&c->aux[3], total.units);
+    if (a.trace) atomicMax(a.trace + 5, global_ns());  // the last CTA to finish
   }
-  if (!t.sync()) return false;
-  {
-    uint32_t o_e = 0, o_m = 0, t_e = 0, t_m = 0;
-    for (uint32_t j = tid; j < nb; j += blockDim.x) {
-      const uint32_t pe = ld_cg(a.part + 2 * nb + 2 * j), pm = ld_cg(a.part + 2 * nb + 2 * j + 1);
-      t_e += pe;
-      t_m += pm;
-      if (j < b) {
-        o_e += pe;
-        o_m += pm;
-      }
-    }
-    block_sum4(o_e, o_m, t_e, t_m);
-    if (b == 0 && tid == 0) {
-      c->aux[2] = t_e;
-      c->aux[3] = t_m;
-    }
-    if (t_e > a.ecap || (unsigned long long)t_m * a.QW > a.mcap) {
-      if (tid == 0) set_err(c, a.qerr, kErrInternal);
-      return false;
-    }
-    for (uint32_t base = rlo; base < rhi; base += blockDim.x) {
-      const uint32_t r = base + tid;
-      uint32_t f = 0, m = 0;
-      if (r < rhi) {
-        f = ld_cg(a.qcnt + 2 * r);
-        m = ld_cg(a.qcnt + 2 * r + 1);
-      }
-      uint32_t ee, em, te, tm;
-      block_excl_scan2(f + m, m, ee, em, te, tm);
-      if (r < rhi) {
-        const uint32_t start = o_e + ee;
-        a.qrow[r] = make_uint4(start, start + f, o_m + em, start + f + m);
-        a.cur[2 * r] = start;
-        a.cur[2 * r + 1] = start + f;
-      }
-      o_e += te;
-      o_m += tm;
-    }
-  }
-  if (!t.sync()) return false;
-
-  // ---- P5: fill
-  if (a.trace && b == 0 && tid == 0) a.trace[4] = global_ns();
-  qrs_walk<true>(a, t, NU, U0, &c->ticket[1]);
-  if (a.trace && tid == 0) atomicMax(a.trace + 5, global_ns());  // the last CTA to finish
   return true;
 }
 

@@ -140,7 +140,7 @@ __device__ bool relax_team(const RelaxArgs& a, const Team& t, StageMem* stage) {
           const uint4 d = a.qrow[px];
           if (atomicExch(a.stamp + px, 1u) != 1u) {
             push = true;
-            deg = d.w - d.x;
+            deg = d.z + d.w;
           }
         }
         stage_push_units(push, px, deg, a.cshift, st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
@@ -179,7 +179,8 @@ __device__ bool relax_team(const RelaxArgs& a, const Team& t, StageMem* stage) {
     const Batches bt{n, (uint32_t)G, nwarps, gwarp, &c->ticket[cur]};
     for (uint32_t t0 = bt.first(); t0 < n; t0 = bt.next(lane)) {
       const uint32_t ui = t0 + grp;
-      uint32_t beg = 0, end = 0, fe = 0, nfb = 0;
+      uint32_t beg = 0, end = 0;  // of the unit, counted over the row's all-window edges and then the others
+      uint4 d = make_uint4(0u, 0u, 0u, 0u);
       bool q1 = false;  // the unit's row belongs to the second query
       uint32_t sv[K];
 #pragma unroll
@@ -188,11 +189,9 @@ __device__ bool relax_team(const RelaxArgs& a, const Team& t, StageMem* stage) {
         const unsigned long long u = qin[ui];  // written before the last barrier
         const uint32_t r = (uint32_t)u, ch = (uint32_t)(u >> 32);
         q1 = r >= U0;
-        const uint4 d = a.qrow[r];
-        beg = d.x + (ch << a.cshift);
-        end = min(d.w, beg + (1u << a.cshift));
-        fe = d.y;
-        nfb = d.z;
+        d = a.qrow[r];
+        beg = ch << a.cshift;
+        end = min(d.z + d.w, beg + (1u << a.cshift));
         const uint32_t* src = a.val + ((size_t)r << lps) + gl;
 #pragma unroll
         for (int kk = 0; kk < K; ++kk) sv[kk] = ld_val(src + kk * P);
@@ -205,11 +204,13 @@ __device__ bool relax_team(const RelaxArgs& a, const Team& t, StageMem* stage) {
         uint32_t xr = 0, w = 0;
         uint64_t m0 = ~0ull, m1 = ~0ull;
         if (e < end) {
-          const uint2 ew = a.qcw[e];
+          const bool full = e < d.z;
+          const uint32_t k = full ? d.x + e : d.y + (e - d.z);
+          const uint2 ew = (full ? a.qcw : a.qmcw)[k];
           xr = ew.x;
           w = ew.y;
-          if (e >= fe) {
-            const uint64_t* mp = a.qmask + (size_t)(nfb + (e - fe)) * a.QW;
+          if (!full) {
+            const uint64_t* mp = a.qmask + (size_t)k * a.QW;
             m0 = mask_extract(mp, a.QW, a.s0);
             if (P * K > 64) m1 = mask_extract(mp, a.QW, a.s0 + 64u);
           }
@@ -275,10 +276,10 @@ __device__ bool relax_team(const RelaxArgs& a, const Team& t, StageMem* stage) {
         bool push = false;
         uint32_t deg = 0;
         if (pend) {
-          const uint4 d = a.qrow[pend_x];  // issued alongside the stamp exchange
+          const uint4 dx = a.qrow[pend_x];  // issued alongside the stamp exchange
           if (atomicExch(a.stamp + pend_x, stamp_next) != stamp_next) {
             push = true;
-            deg = d.w - d.x;
+            deg = dx.z + dx.w;
           }
         }
         stage_push_units(push, pend_x, deg, a.cshift, st, qout, qn_out, a.qcap, c, a.qerr, lane);
