@@ -505,6 +505,7 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
       (st = alloc_n(c, c->scratch_bufs, qcap, &c->q0)) || (st = alloc_n(c, c->scratch_bufs, qcap, &c->q1)) ||
       (st = alloc_n(c, c->scratch_bufs, ucap, &c->units)) ||
       (st = alloc_n(c, c->scratch_bufs, kNumCtl, &c->ctl)) || (st = alloc_n(c, c->scratch_bufs, 1, &c->qerr)) ||
+      (st = alloc_n(c, c->scratch_bufs, 6 * kBestSnaps, &c->rbest)) ||
       (st = alloc_n(c, c->scratch_bufs, (uint64_t)V + (E2 >> 4) + 64, &c->procv))) {
     free_graph(c);
     return st;
@@ -687,6 +688,7 @@ svv_status enqueue_tail(svv_ctx* c, int t, uint32_t wb, uint32_t wl, uint32_t* o
     r.qmcw = c->qmcw;
     r.qmask = c->qmask;
     r.counts = &(c->ctl + 2)->aux[0];
+    r.best = c->rbest;
     r.val = c->val;
     r.LP = P * K;
     r.stamp = c->stamp;

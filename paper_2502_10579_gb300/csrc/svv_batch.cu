@@ -163,6 +163,7 @@ __device__ bool run_instance(const BatchArgs& b, const BatchInstance& q, uint32_
     x.qmcw = sc.qmcw;
     x.qmask = sc.qmask;
     x.counts = &(tc + 3)->aux[0];
+    x.best = sc.rbest;
     x.val = sc.val;
     x.LP = P * K;
     x.stamp = sc.stamp;

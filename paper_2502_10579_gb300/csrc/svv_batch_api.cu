@@ -21,7 +21,7 @@ static uint64_t team_bytes(const svv_ctx* c, uint32_t LP, uint32_t QW, uint32_t 
   const uint64_t ucap = V + E / (1u << c->qrs_cs) + 64;
   uint64_t b = 0;
   b += 5 * round256(V * 4);                  // rI, rU, stamp, row, uv
-  b += round256(8ull * team_blocks * 4);     // part
+  b += round256(8ull * team_blocks * 4) + round256(6 * kBestSnaps * 4);  // part, rbest
   b += round256(V * 16);                     // qrow
   b += round256(E * 8);                      // qcw
   b += round256(NF * 8) + round256(NF * QW * 8);  // qmcw, qmask
@@ -40,6 +40,7 @@ static svv_status alloc_team(svv_ctx* c, std::vector<void*>& owner, uint32_t LP,
   if ((st = alloc_n(c, owner, V, &t.rI)) || (st = alloc_n(c, owner, V, &t.rU)) ||
       (st = alloc_n(c, owner, V, &t.stamp)) || (st = alloc_n(c, owner, V, &t.row)) ||
       (st = alloc_n(c, owner, V, &t.uv)) || (st = alloc_n(c, owner, 8ull * team_blocks, &t.part)) ||
+      (st = alloc_n(c, owner, 6 * kBestSnaps, &t.rbest)) ||
       (st = alloc_n(c, owner, V, &t.qrow)) || (st = alloc_n(c, owner, E, &t.qcw)) ||
       (st = alloc_n(c, owner, NF, &t.qmcw)) ||
       (st = alloc_n(c, owner, NF * QW, &t.qmask)) || (st = alloc_n(c, owner, V * LP, &t.val)) ||

@@ -170,7 +170,7 @@ struct svv_ctx {
   // query scratch (sized at load from V and E; the L-dependent part on demand)
   std::vector<void*> scratch_bufs;
   uint32_t *rI = nullptr, *rU = nullptr, *stamp = nullptr, *row = nullptr, *uv = nullptr;
-  uint32_t *part = nullptr, *qerr = nullptr;
+  uint32_t *part = nullptr, *qerr = nullptr, *rbest = nullptr;
   uint4* qrow = nullptr;
   uint2 *qcw = nullptr, *qmcw = nullptr;
   unsigned long long *q0 = nullptr, *q1 = nullptr, *units = nullptr;

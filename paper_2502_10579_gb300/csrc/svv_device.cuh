@@ -228,9 +228,8 @@ struct OpSSSP {  // CASMIN(Val(v), Val(u) + w), saturating
   static constexpr uint32_t kIdentity = kInf;
   static constexpr uint32_t kSource = 0;
   __device__ __forceinline__ static uint32_t relax(uint32_t sv, uint32_t w) {
-    if (sv == kInf) return kInf;
-    unsigned long long s = (unsigned long long)sv + w;
-    return s > kSat ? kSat : (uint32_t)s;
+    const uint32_t s = sv + w;
+    return sv == kInf ? kInf : (s < w || s > kSat) ? kSat : s;
   }
   __host__ __device__ __forceinline__ static constexpr bool better(uint32_t a, uint32_t b) { return a < b; }
   __device__ __forceinline__ static uint32_t atomic(uint32_t* p, uint32_t v) { return atomicMin(p, v); }
@@ -291,8 +290,8 @@ struct OpMixed {
   __device__ __forceinline__ static uint32_t relax_kind(uint32_t kind, uint32_t sv, uint32_t w) {
     if (sv == kInf) return kInf;
     if (kind == kKindSum) {
-      const unsigned long long s = (unsigned long long)sv + w;
-      return s > kSat ? kSat : (uint32_t)s;
+      const uint32_t s = sv + w;
+      return (s < w || s > kSat) ? kSat : s;
     }
     if (kind == kKindHop) return sv + 1u;
     const uint32_t x = kind == kKindMax ? w : ~w;

@@ -86,7 +86,7 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, StageMem* st
   // over all of them
   const unsigned gwarp = (threadIdx.x >> 5) * t.nblocks + t.rank, nwarps = nthreads >> 5;
   if (a.qerr && cta_read(a.qerr) != 0u) return false;
-  PushStage st(stage);
+  PushStage st(stage, true);
   // The best improved value of every round goes to a ring as in the single
   // solve: one for the whole group (a bound for each of its lanes), or one per
   // lane for the two lanes of a mixed pair, whose values do not compare.

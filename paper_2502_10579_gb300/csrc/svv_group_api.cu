@@ -269,6 +269,7 @@ svv_status enqueue_pair_tail(svv_ctx* c, const BatchInstance* inst, uint32_t* co
   r.qmask = c->p_qmask;
   r.counts = &(c->ctl + 2)->aux[0];
   r.counts1 = &(c->ctl + 6)->aux[0];
+  r.best = c->rbest;
   if (mixed) {
     r.kind0 = kind_of(inst[0].type);
     r.kind1 = kind_of(inst[1].type);

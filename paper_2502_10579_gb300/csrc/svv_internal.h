@@ -154,6 +154,7 @@ struct QrsArgs {
   unsigned int* counts1_out;
 };
 
+constexpr uint32_t kBestSnaps = 128;  // snapshots of the longest slab
 struct RelaxArgs {
   DevGraph g;
   Window win;
@@ -177,6 +178,9 @@ struct RelaxArgs {
   // a pair of different types (OpMixed): each query's relaxation kind, and
   // bit q set when query q's rows hold complemented values (SSWP)
   uint32_t kind0, kind1, flip;
+  // [3][2][kBestSnaps] scratch: per round (a ring), query and snapshot, the
+  // best value (nf_key, 0: none) that the round before gave a row
+  uint32_t* best;
   uint32_t* val;          // [U * LP]
   uint32_t LP;            // row stride of val (>= ls)
   uint32_t* stamp;        // [V]
@@ -242,7 +246,7 @@ struct BatchInstance {
 
 // per-team query scratch (same roles as the single-query scratch)
 struct TeamScratch {
-  uint32_t *rI, *rU, *stamp, *row, *uv, *part;
+  uint32_t *rI, *rU, *stamp, *row, *uv, *part, *rbest;
   uint4* qrow;
   uint2 *qcw, *qmcw;
   uint64_t* qmask;

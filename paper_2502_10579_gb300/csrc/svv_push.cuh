@@ -58,6 +58,8 @@ constexpr int kStageThreads = 512;  // of every kernel that stages pushes
 struct StageMem {  // a kernel's shared memory for staged pushes
   unsigned long long units[(kStageThreads / 32) * kStageUnits];
   StageHubs hubs;
+  uint32_t best[2][kBestSnaps];  // the relaxation's, here so that its instances share it
+  uint32_t changed;              // improvements of a pull round
 };
 
 struct PushStage {
@@ -65,9 +67,11 @@ struct PushStage {
   uint32_t fill;            // warp-uniform
   uint32_t out;             // units this warp copied to the queue in this round (warp-uniform)
   StageHubs* hubs;
-  __device__ __forceinline__ explicit PushStage(StageMem* m)  // a CTA barrier comes before the first push
+  // `fresh`: the first stage of the kernel on this memory (a CTA barrier comes
+  // before its first push); else everything staged before has been flushed
+  __device__ __forceinline__ PushStage(StageMem* m, bool fresh)
       : buf(m->units + (threadIdx.x >> 5) * kStageUnits), fill(0u), out(0u), hubs(&m->hubs) {
-    if (threadIdx.x == 0) m->hubs.n = 0u;
+    if (fresh && threadIdx.x == 0) m->hubs.n = 0u;
   }
 };
 

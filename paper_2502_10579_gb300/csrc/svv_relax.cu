@@ -28,7 +28,7 @@ namespace svv {
 constexpr int kRelaxThreads = kStageThreads;
 
 template <class Op, int P, int K>
-__global__ void __launch_bounds__(kRelaxThreads, 2) relax_kernel(RelaxArgs a) {
+__global__ void __launch_bounds__(kRelaxThreads, 2) relax_kernel(const __grid_constant__ RelaxArgs a) {
   __shared__ StageMem s_stage;
   __shared__ TeamBar s_bar;
   const Team t{a.ctl, a.qerr, gridDim.x, blockIdx.x, a.spin_ns, &s_bar};

@@ -19,7 +19,7 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, StageMem* stage) {
   // over all of them
   const unsigned gwarp = (threadIdx.x >> 5) * t.nblocks + t.rank, nwarps = nthreads >> 5;
   if (a.qerr && cta_read(a.qerr) != 0u) return false;
-  PushStage st(stage);
+  PushStage st(stage, true);
   __shared__ uint32_t s_changed, s_key;  // this CTA's improvements of a round, and the best of them
   if (threadIdx.x == 0) s_changed = s_key = 0u;
 

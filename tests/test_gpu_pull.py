@@ -84,6 +84,34 @@ def test_pull_rounds(svv, V, kind):
                 np.testing.assert_array_equal(svv.to_u32(out), want[t, b, L])
 
 
+@pytest.mark.parametrize("kind", list(WEIGHTS))
+@pytest.mark.parametrize("V", [33, 1025, 5000])
+def test_relaxation_pull_rounds(svv, V, kind):
+    """Without pruning every vertex has a row and most rows change at once, so
+    the relaxation's rounds pull: rows of 32, 64 and 128 values, slabs, one query
+    and pairs (one type and several), every type."""
+    log = make_log(V, WEIGHTS[kind], seed=V + 1)
+    lens = [17, 32, 33, 64, 65, 70]
+    with svv.Context(0) as ctx:
+        ctx.set_tuning("prune", 0)
+        ctx.set_tuning("batch_mode", 2)
+        ctx.set_tuning("group_mix", 1)
+        ctx.load_log(log)
+        want = {t: oracle.query(log, t, 0, 0, log.S) for t in range(4)}
+        for L in lens:
+            for t in range(4):
+                b = (3 * t) % (log.S - L + 1)
+                np.testing.assert_array_equal(svv.to_u32(ctx.query(t, 0, b, L)), want[t][b:b + L])
+            for t0, t1 in [(0, 0), (1, 1), (0, 1), (2, 3), (1, 2)]:
+                b = (log.S - L) // 2
+                outs, status = ctx.query_batch([(t0, 0, 0, L), (t1, 0, b, L)])
+                assert status == [0, 0]
+                np.testing.assert_array_equal(svv.to_u32(outs[0]), want[t0][:L])
+                np.testing.assert_array_equal(svv.to_u32(outs[1]), want[t1][b:b + L])
+        ctx.set_tuning("slab_max", 40)
+        np.testing.assert_array_equal(svv.to_u32(ctx.query(0, 0, 0, log.S)), want[0])
+
+
 def test_source_far_from_targets(svv):
     """Most targets unreachable: nothing ends early, every in-edge is looked at."""
     log = make_log(3000, WEIGHTS["small"], seed=9)
