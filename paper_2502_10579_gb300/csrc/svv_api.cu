@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "svv_ctx.h"
+#include "svv_threads.h"
 
 using namespace svv;
 
@@ -393,55 +394,74 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
   }
   // validate
   if (row_ptr[0] != 0) return fail(c, SVV_EINVAL, "row_ptr[0] != 0");
-  for (uint32_t v = 0; v < V; ++v)
-    if (row_ptr[v + 1] < row_ptr[v]) return fail(c, SVV_EINVAL, "row_ptr not non-decreasing");
+  const unsigned nt = host_threads(std::max<uint64_t>(V, E));
+  std::vector<char> bad_row(nt, 0), bad_col(nt, 0);
+  parallel(nt, [&](unsigned t) {
+    bool bad = false;
+    for (uint64_t v = part(V, nt, t), hi = part(V, nt, t + 1); v < hi; ++v) bad |= row_ptr[v + 1] < row_ptr[v];
+    bad_row[t] = bad;
+  });
+  if (std::count(bad_row.begin(), bad_row.end(), 0) != (long)nt) return fail(c, SVV_EINVAL, "row_ptr not non-decreasing");
   if (row_ptr[V] != E) return fail(c, SVV_EINVAL, "row_ptr[V] != E");
-  for (uint64_t e = 0; e < E; ++e)
-    if (col[e] >= V) return fail(c, SVV_EINVAL, "col >= V");
+  parallel(nt, [&](unsigned t) {
+    bool bad = false;
+    for (uint64_t e = part(E, nt, t), hi = part(E, nt, t + 1); e < hi; ++e) bad |= col[e] >= V;
+    bad_col[t] = bad;
+  });
+  if (std::count(bad_col.begin(), bad_col.end(), 0) != (long)nt) return fail(c, SVV_EINVAL, "col >= V");
 
-  // classify against the history [0, S): full / partial / absent
+  // classify against the history [0, S): full / partial / absent; threads take
+  // ranges of rows with equal numbers of edges
   std::vector<uint64_t> hist(W);
   for (uint32_t j = 0; j < W; ++j) {
     const uint32_t n = std::min<uint32_t>(64, S - 64 * j);
     hist[j] = n == 64 ? ~0ull : ((1ull << n) - 1ull);
   }
   std::vector<uint32_t> rp((size_t)V + 1, 0), nfp((size_t)V + 1, 0);
-  std::vector<uint8_t> kind(E);  // 0 absent, 1 full, 2 partial
-  for (uint32_t v = 0; v < V; ++v) {
-    uint32_t nfull = 0, npart = 0;
-    for (uint64_t e = row_ptr[v]; e < row_ptr[v + 1]; ++e) {
-      bool all = true, any = false;
-      const uint64_t* m = mask + e * W;
-      for (uint32_t j = 0; j < W; ++j) {
-        const uint64_t x = m[j] & hist[j];
-        all &= (x == hist[j]);
-        any |= (x != 0);
+  std::unique_ptr<uint8_t[]> kind(new uint8_t[std::max<uint64_t>(E, 1)]);  // 0 absent, 1 full, 2 partial
+  parallel(nt, [&](unsigned t) {
+    for (uint64_t v = row_at(row_ptr, V, nt, t), hi = row_at(row_ptr, V, nt, t + 1); v < hi; ++v) {
+      uint32_t nfull = 0, npart = 0;
+      for (uint64_t e = row_ptr[v]; e < row_ptr[v + 1]; ++e) {
+        bool all = true, any = false;
+        const uint64_t* m = mask + e * W;
+        for (uint32_t j = 0; j < W; ++j) {
+          const uint64_t x = m[j] & hist[j];
+          all &= (x == hist[j]);
+          any |= (x != 0);
+        }
+        kind[e] = all ? 1 : (any ? 2 : 0);
+        nfull += all;
+        npart += (!all && any);
       }
-      kind[e] = all ? 1 : (any ? 2 : 0);
-      nfull += all;
-      npart += (!all && any);
+      rp[v + 1] = nfull + npart;
+      nfp[v + 1] = npart;
     }
-    rp[v + 1] = rp[v] + nfull + npart;
-    nfp[v + 1] = nfp[v] + npart;
+  });
+  for (uint32_t v = 0; v < V; ++v) {
+    rp[v + 1] += rp[v];
+    nfp[v + 1] += nfp[v];
   }
   const uint32_t E2 = rp[V], NF = nfp[V];
-  std::vector<uint2> cw(std::max<uint32_t>(E2, 1)), nfcw(std::max<uint32_t>(NF, 1));
-  std::vector<uint32_t> nfsrc(std::max<uint32_t>(NF, 1));
-  std::vector<uint64_t> nfm((size_t)std::max<uint32_t>(NF, 1) * W);
-  for (uint32_t v = 0; v < V; ++v) {
-    uint32_t pf = rp[v], pn = rp[v + 1] - (nfp[v + 1] - nfp[v]), k = nfp[v];
-    for (uint64_t e = row_ptr[v]; e < row_ptr[v + 1]; ++e) {
-      if (kind[e] == 1) {
-        cw[pf++] = make_uint2(col[e], weight[e]);
-      } else if (kind[e] == 2) {
-        cw[pn++] = make_uint2(col[e], weight[e]);
-        nfcw[k] = make_uint2(col[e], weight[e]);
-        nfsrc[k] = v;
-        for (uint32_t j = 0; j < W; ++j) nfm[(size_t)k * W + j] = mask[e * W + j] & hist[j];
-        ++k;
+  std::unique_ptr<uint2[]> cw(new uint2[std::max<uint32_t>(E2, 1)]), nfcw(new uint2[std::max<uint32_t>(NF, 1)]);
+  std::unique_ptr<uint32_t[]> nfsrc(new uint32_t[std::max<uint32_t>(NF, 1)]);
+  std::unique_ptr<uint64_t[]> nfm(new uint64_t[(size_t)std::max<uint32_t>(NF, 1) * W]);
+  parallel(nt, [&](unsigned t) {
+    for (uint64_t v = row_at(row_ptr, V, nt, t), hi = row_at(row_ptr, V, nt, t + 1); v < hi; ++v) {
+      uint32_t pf = rp[v], pn = rp[v + 1] - (nfp[v + 1] - nfp[v]), k = nfp[v];
+      for (uint64_t e = row_ptr[v]; e < row_ptr[v + 1]; ++e) {
+        if (kind[e] == 1) {
+          cw[pf++] = make_uint2(col[e], weight[e]);
+        } else if (kind[e] == 2) {
+          cw[pn++] = make_uint2(col[e], weight[e]);
+          nfcw[k] = make_uint2(col[e], weight[e]);
+          nfsrc[k] = (uint32_t)v;
+          for (uint32_t j = 0; j < W; ++j) nfm[(size_t)k * W + j] = mask[e * W + j] & hist[j];
+          ++k;
+        }
       }
     }
-  }
+  });
 
   // replace the resident graph
   cudaDeviceSynchronize();
@@ -474,10 +494,10 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
     return st;
   }
   cudaError_t e = cudaMemcpy(d_rp, rp.data(), rp.size() * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(d_cw, cw.data(), (size_t)E2 * 8, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(d_nfm, nfm.data(), (size_t)NF * W * 8, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(d_nfsrc, nfsrc.data(), (size_t)NF * 4, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(d_nfcw, nfcw.data(), (size_t)NF * 8, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(d_cw, cw.get(), (size_t)E2 * 8, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(d_nfm, nfm.get(), (size_t)NF * W * 8, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(d_nfsrc, nfsrc.get(), (size_t)NF * 4, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(d_nfcw, nfcw.get(), (size_t)NF * 8, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) {
     free_graph(c);
     return cuda_fail(c, e, "uploading the graph");
