@@ -141,11 +141,12 @@ SolveArgs solve_base(svv_ctx* c, uint32_t wb, uint32_t wl, int type, const Knobs
 }
 
 svv_status finish(svv_ctx* c, cudaStream_t s, int nctl_copy) {
-  cudaError_t e = cudaMemcpyAsync(c->hctl, c->ctl, sizeof(TeamCtl) * nctl_copy, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(c->hqerr, c->qerr, sizeof(uint32_t), cudaMemcpyDeviceToHost, s);
+  // the query's error word lives in control block kErrCtl: one copy brings both
+  cudaError_t e = cudaMemcpyAsync(c->hctl, c->ctl, sizeof(TeamCtl) * std::max(nctl_copy, kErrCtl + 1),
+                                  cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(c, e, "query");
-  const uint32_t q = *c->hqerr;
+  const uint32_t q = c->hctl[kErrCtl].err;
   if (q == kErrTimeout) return fail(c, SVV_ETIMEOUT, "a device wait or the round cap expired");
   if (q == 2u) return fail(c, SVV_ENOMEM, "rows_out is smaller than U * win_len");
   if (q != 0) return fail(c, SVV_EINTERNAL, "device capacity check failed");
@@ -210,7 +211,6 @@ svv_status svv_create(svv_ctx** out, int device, uint64_t budget) {
     return SVV_ECUDA;
   }
   e = cudaMallocHost((void**)&c->hctl, sizeof(TeamCtl) * kNumCtl);
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&c->hqerr, sizeof(uint32_t));
   if (e != cudaSuccess) {
     if (c->hctl) cudaFreeHost(c->hctl);
     delete c;
@@ -228,7 +228,6 @@ void svv_destroy(svv_ctx* c) {
     cudaDeviceSynchronize();
     free_graph(c);
     if (c->hctl) cudaFreeHost(c->hctl);
-    if (c->hqerr) cudaFreeHost(c->hqerr);
     for (auto& e : c->ev)
       if (e) cudaEventDestroy(e);
     for (auto& e : c->bev)
@@ -524,12 +523,13 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
       (st = alloc_n(c, c->scratch_bufs, std::max<uint32_t>(NF, 1), &c->qmcw)) ||
       (st = alloc_n(c, c->scratch_bufs, qcap, &c->q0)) || (st = alloc_n(c, c->scratch_bufs, qcap, &c->q1)) ||
       (st = alloc_n(c, c->scratch_bufs, ucap, &c->units)) ||
-      (st = alloc_n(c, c->scratch_bufs, kNumCtl, &c->ctl)) || (st = alloc_n(c, c->scratch_bufs, 1, &c->qerr)) ||
+      (st = alloc_n(c, c->scratch_bufs, kNumCtl, &c->ctl)) ||
       (st = alloc_n(c, c->scratch_bufs, 6 * kBestSnaps, &c->rbest)) ||
       (st = alloc_n(c, c->scratch_bufs, (uint64_t)V + (E2 >> 4) + 64, &c->procv))) {
     free_graph(c);
     return st;
   }
+  c->qerr = &c->ctl[kErrCtl].err;
   c->qcap = (uint32_t)qcap;
   c->ucap = (uint32_t)ucap;
   c->pcap = (uint32_t)((uint64_t)V + (E2 >> 4) + 64);
@@ -600,8 +600,7 @@ svv_status enqueue_query(svv_ctx* c, int t, uint32_t source, uint32_t wb, uint32
                          cudaStream_t s, bool timing, float* ms_relax_out, float* ms_scatter_out,
                          const CompactOut* co) {
   *ms_relax_out = *ms_scatter_out = 0.f;
-  cudaError_t e = cudaMemsetAsync(c->ctl, 0, sizeof(TeamCtl) * 8, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->qerr, 0, sizeof(uint32_t), s);
+  cudaError_t e = cudaMemsetAsync(c->ctl, 0, sizeof(TeamCtl) * 8, s);  // the error word too
   if (e != cudaSuccess) return cuda_fail(c, e, "memset");
   if (timing) cudaEventRecord(c->ev[0], s);
   if (source_is_isolated(c, source)) return enqueue_isolated(c, t, source, wl, out, s, timing, co);
@@ -969,10 +968,7 @@ svv_status batch_in_order(svv_ctx* c, const BatchInstance* inst, uint32_t m, con
         const uint32_t* pI[2] = {c->gI[0], c->gI[1]};
         const uint32_t* pU[2] = {c->gU[0], c->gU[1]};
         bool done = false;
-        if ((e = cudaMemcpyAsync(c->qerr, c->gerr, sizeof(uint32_t), cudaMemcpyDeviceToDevice, es)) != cudaSuccess)
-          st = cuda_fail(c, e, "group status copy");
-        else
-          st = enqueue_pair_tail(c, gi, po, pI, pU, es, &done);
+        st = enqueue_pair_tail(c, gi, po, pI, pU, es, &done);  // goes on from the bounds' error word
         if (st) return capture ? end_capture(st) : st;
         if (done) {
           for (int j = 0; j < 2; ++j)

@@ -16,7 +16,8 @@
 
 namespace svv {
 
-constexpr int kNumCtl = 8 + 256;  // 0..3 query phases, 4..5 group solves, 8.. per-snapshot plain solves
+constexpr int kNumCtl = 8 + 256;  // 0..3 query phases, 4..5 group solves, 6 a pair's second count, 8.. plain solves
+constexpr int kErrCtl = 7;        // its err is the query-wide error word
 constexpr int kAsyncSlots = 64;   // svv_query_async queries in flight
 constexpr uint32_t kMaxSlab = 128;
 constexpr uint32_t kTraceCap = 4096;
@@ -177,7 +178,6 @@ struct svv_ctx {
   uint32_t qcap = 0, ucap = 0, ecap = 0;
   svv::TeamCtl* ctl = nullptr;
   svv::TeamCtl* hctl = nullptr;  // pinned mirror
-  uint32_t* hqerr = nullptr;
   // window-dependent
   uint64_t* qmask = nullptr;
   uint64_t mcap = 0;

@@ -60,8 +60,8 @@ svv_status enqueue_group_bounds(svv_ctx* c, int t, const BatchInstance* inst, ui
     }
   }
   const int gt = mixed ? kTypeMixed : t;
-  cudaError_t e = cudaMemsetAsync(c->ctl + 4, 0, sizeof(TeamCtl) * 2, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->qerr, 0, sizeof(uint32_t), s);
+  // the group's blocks, those of a pair tail that follows, and the error word
+  cudaError_t e = cudaMemsetAsync(c->ctl + 2, 0, sizeof(TeamCtl) * (kErrCtl - 1), s);
   if (e != cudaSuccess) return cuda_fail(c, e, "memset");
 
   LanesArgs la{};
@@ -210,9 +210,7 @@ svv_status enqueue_pair_tail(svv_ctx* c, const BatchInstance* inst, uint32_t* co
   svv_status st = ensure_pair_rows(c, P * K);
   if (st) return st;
   if (c->p_qcap > 0xFFFFFFFFull) return SVV_OK;
-  cudaError_t e = cudaMemsetAsync(c->ctl + 2, 0, sizeof(TeamCtl) * 2, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(c->ctl + 6, 0, sizeof(TeamCtl), s);
-  if (e != cudaSuccess) return cuda_fail(c, e, "memset");
+  cudaError_t e = cudaSuccess;  // its control blocks were cleared with the group's
   c->last_rI = rI[1];  // svv_get_bounds: the batch's last instance
   c->last_rU = rU[1];
   c->last_row = c->p_row1;
