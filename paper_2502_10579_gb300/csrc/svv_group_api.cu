@@ -205,6 +205,9 @@ svv_status enqueue_pair_tail(svv_ctx* c, const BatchInstance* inst, uint32_t* co
   if (wl > std::max<uint32_t>(1, std::min(k0.slab_max, kMaxSlab)) ||
       wl > std::max<uint32_t>(1, std::min(k1.slab_max, kMaxSlab)) || k0.relax_lanes != k1.relax_lanes)
     return SVV_OK;
+  // a row has room for all its out-edges: both queries' rows and edges are
+  // counted in 32 bits
+  if (2 * std::max<uint64_t>(c->ecap, c->g.V) > 0xFFFFFFFFull) return SVV_OK;
   uint32_t P, K;
   slab_shape_p(wl, k0.relax_lanes, P, K);
   svv_status st = ensure_pair_rows(c, P * K);

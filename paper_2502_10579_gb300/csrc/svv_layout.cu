@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(256) rekey_kernel(DevGraph g, int part, uint2*
 // per block (blocks take consecutive ranges), their exclusive scan in digit
 // order, and the ordered move.
 __device__ __forceinline__ void sort_range(uint32_t n, uint32_t& lo, uint32_t& hi) {
-  const uint32_t per = (n + gridDim.x - 1u) / gridDim.x;
+  const uint32_t per = n / gridDim.x + (n % gridDim.x != 0u);  // n may be close to 2^32
   lo = (uint32_t)min((unsigned long long)n, (unsigned long long)per * blockIdx.x);
   hi = (uint32_t)min((unsigned long long)n, (unsigned long long)per * blockIdx.x + per);
 }

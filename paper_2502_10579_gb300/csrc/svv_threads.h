@@ -3,7 +3,6 @@
 
 #include <algorithm>
 #include <cstdint>
-#include <system_error>
 #include <thread>
 #include <vector>
 
@@ -23,7 +22,7 @@ void parallel(unsigned n, F f) {
   try {
     th.reserve(n);
     for (; started + 1 < n; ++started) th.emplace_back(f, started);
-  } catch (const std::system_error&) {  // no more threads: the rest runs here
+  } catch (...) {  // no more threads or no memory for one: the rest runs here
   }
   for (unsigned t = started; t < n; ++t) f(t);
   for (auto& t : th) t.join();
