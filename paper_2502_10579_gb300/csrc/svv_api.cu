@@ -514,10 +514,9 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
     free_graph(c);
     return fail(c, SVV_EINVAL, "graph too large for 32-bit work queues");
   }
-  const uint64_t nblk = (uint64_t)c->num_sms * 4;
   if ((st = alloc_n(c, c->scratch_bufs, V, &c->rI)) || (st = alloc_n(c, c->scratch_bufs, V, &c->rU)) ||
       (st = alloc_n(c, c->scratch_bufs, V, &c->stamp)) || (st = alloc_n(c, c->scratch_bufs, V, &c->row)) ||
-      (st = alloc_n(c, c->scratch_bufs, V, &c->uv)) || (st = alloc_n(c, c->scratch_bufs, 8 * nblk, &c->part)) ||
+      (st = alloc_n(c, c->scratch_bufs, V, &c->uv)) || (st = alloc_n(c, c->scratch_bufs, part_words(c->num_sms), &c->part)) ||
       (st = alloc_n(c, c->scratch_bufs, V, &c->qrow)) ||
       (st = alloc_n(c, c->scratch_bufs, std::max<uint32_t>(E2, 1), &c->qcw)) ||
       (st = alloc_n(c, c->scratch_bufs, std::max<uint32_t>(NF, 1), &c->qmcw)) ||

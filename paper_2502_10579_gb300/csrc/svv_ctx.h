@@ -306,6 +306,10 @@ svv_status alloc_n(svv_ctx* c, std::vector<void*>& owner, uint64_t n, T** out) {
 
 inline uint32_t ceil_div(uint64_t a, uint64_t b) { return (uint32_t)((a + b - 1) / b); }
 
+// words of a context's per-CTA sums: 8 for each of up to 4 CTAs per SM, and on a
+// device of few SMs (a partition) as many as the layout builder's counters take
+inline uint64_t part_words(int num_sms) { return std::max<uint64_t>(8ull * 4ull * (uint64_t)num_sms, kLayoutWords); }
+
 // lanes per edge P and snapshots per lane K for a slab of ls snapshots, with
 // at most max_p lanes per edge (P*K is the padded row length)
 inline void slab_shape_p(uint32_t ls, uint32_t max_p, uint32_t& P, uint32_t& K) {

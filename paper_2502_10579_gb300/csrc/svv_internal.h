@@ -46,6 +46,9 @@ static_assert(sizeof(TeamCtl) % 128 == 0, "TeamCtl must be cache-line sized");
 // slots {source, weight} of row first + k, one per target.  The first nhub
 // slices hold one target each, its in-edges over all lanes.
 constexpr uint32_t kItemSteps = 16;
+// counters of the layout builder (words); they live in the per-CTA sums of the
+// extraction, see part_words
+constexpr uint32_t kLayoutWords = 1068;
 struct PullGraph {
   const uint2* items;
   const uint32_t* tgt;
@@ -129,7 +132,7 @@ struct QrsArgs {
   const uint32_t* rU;     // union-graph values
   uint32_t* row;          // [V] vertex -> row, kNone if stable
   uint32_t* uv;           // [V] row -> vertex
-  uint32_t* part;         // [8 * gridDim] per-CTA sums
+  uint32_t* part;         // [8 * gridDim] per-CTA sums (part_words)
   unsigned long long* units;  // row | chunk << 32 over unstable rows
   uint32_t ucap;
   uint32_t cshift;

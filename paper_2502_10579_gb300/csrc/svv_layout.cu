@@ -356,8 +356,9 @@ svv_status build_pull(svv_ctx* c) {
   uint32_t* sitem = reinterpret_cast<uint32_t*>(c->q0);
   uint2* tpos = reinterpret_cast<uint2*>(c->qrow);
   unsigned long long* meta = reinterpret_cast<unsigned long long*>(c->part);
-  uint32_t *hist = c->part + 2 * kMeta, *off = hist + kBins;  // part holds 32 words per SM
+  uint32_t *hist = c->part + 2 * kMeta, *off = hist + kBins;
   uint32_t* segoff = off + kBins;
+  static_assert(2 * kMeta + 2 * kBins + kMaxSegs == kLayoutWords, "part_words");
   uint32_t* counts = reinterpret_cast<uint32_t*>(c->ctl);  // cleared by every query
   static_assert(sizeof(TeamCtl) * kNumCtl >= 256 * kSortBlocks * sizeof(uint32_t), "sort counters");
   auto step = [&](cudaError_t r) {
