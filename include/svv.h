@@ -108,7 +108,7 @@ svv_status svv_create(svv_ctx **ctx, int device, uint64_t hbm_budget_bytes);
  * Inputs are host arrays of n_inst entries; outputs are caller-owned host
  * arrays: row_ptr[V+1], col[n_inst], weight[n_inst], mask[n_inst*ceil(S/64)].
  * *E_out receives the number of edges written.  SVV_EINVAL on src/dst >= V,
- * S == 0 or t_add/t_del > S. */
+ * S == 0 or t_add/t_del > S; SVV_ENOMEM if host memory runs out. */
 svv_status svv_build_versioned_csr(uint32_t V, uint32_t S, uint64_t n_inst, const uint32_t *src,
                                    const uint32_t *dst, const uint32_t *w, const uint32_t *t_add,
                                    const uint32_t *t_del, uint64_t *row_ptr, uint32_t *col,
@@ -125,7 +125,8 @@ svv_status svv_build_versioned_csr(uint32_t V, uint32_t S, uint64_t n_inst, cons
  * of partial edges) is kept as well for the solves' pull rounds.  Replaces any
  * graph loaded before.
  * SVV_EINVAL on a malformed CSR, S == 0, V >= 2^32-1 or E >= 2^32;
- * SVV_ENOMEM if the resident graph does not fit the budget. */
+ * SVV_ENOMEM if the resident graph does not fit the budget, or (the graph
+ * loaded before then stays) if host memory runs out. */
 svv_status svv_load(svv_ctx *ctx, uint32_t V, uint64_t E, uint32_t S, const uint64_t *row_ptr,
                     const uint32_t *col, const uint32_t *weight, const uint64_t *mask,
                     int inputs_on_device);

@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -362,9 +363,10 @@ svv_status svv_get_stats(svv_ctx* c, svv_stats* out) {
   return SVV_OK;
 }
 
-svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64_t* row_ptr,
-                    const uint32_t* col, const uint32_t* weight, const uint64_t* mask,
-                    int inputs_on_device) {
+// svv_load, but for host memory that runs out (std::bad_alloc)
+static svv_status load_graph(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64_t* row_ptr,
+                             const uint32_t* col, const uint32_t* weight, const uint64_t* mask,
+                             int inputs_on_device) {
   if (!c) return SVV_EINVAL;
   if (V == 0 || V >= 0xFFFFFFFFu) return fail(c, SVV_EINVAL, "V must be in [1, 2^32-2]");
   if (S == 0) return fail(c, SVV_EINVAL, "S must be >= 1");
@@ -546,6 +548,21 @@ svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64
   c->stats = svv_stats{};
   c->err.clear();
   return SVV_OK;
+}
+
+svv_status svv_load(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, const uint64_t* row_ptr,
+                    const uint32_t* col, const uint32_t* weight, const uint64_t* mask,
+                    int inputs_on_device) {
+  try {
+    return load_graph(c, V, E, S, row_ptr, col, weight, mask, inputs_on_device);
+  } catch (const std::bad_alloc&) {
+    // before the resident graph was given up it is still there, untouched
+    if (!c->loaded) {
+      DeviceGuard dg(c->device);
+      free_graph(c);
+    }
+    return fail(c, SVV_ENOMEM, "out of memory");
+  }
 }
 
 }  // extern "C"

@@ -9,15 +9,17 @@
 // instances: 60 ms on one thread).  The ranges of the writing pass hold equal
 // numbers of edges, since low vertex ids carry most of an RMAT graph.
 #include <cstdint>
+#include <new>
 #include <vector>
 
 #include "../../include/svv.h"
 #include "svv_threads.h"
 
-extern "C" svv_status svv_build_versioned_csr(uint32_t V, uint32_t S, uint64_t n_inst, const uint32_t* src,
-                                              const uint32_t* dst, const uint32_t* w, const uint32_t* t_add,
-                                              const uint32_t* t_del, uint64_t* row_ptr, uint32_t* col,
-                                              uint32_t* weight, uint64_t* mask, uint64_t* E_out) {
+// svv_build_versioned_csr, but for memory that runs out (std::bad_alloc)
+static svv_status build_versioned_csr(uint32_t V, uint32_t S, uint64_t n_inst, const uint32_t* src,
+                                      const uint32_t* dst, const uint32_t* w, const uint32_t* t_add,
+                                      const uint32_t* t_del, uint64_t* row_ptr, uint32_t* col,
+                                      uint32_t* weight, uint64_t* mask, uint64_t* E_out) {
   if (V == 0 || S == 0 || !row_ptr || !E_out) return SVV_EINVAL;
   if (n_inst && (!src || !dst || !w || !t_add || !t_del || !col || !weight || !mask)) return SVV_EINVAL;
   const uint32_t W = (S + 63) / 64;
@@ -66,4 +68,15 @@ extern "C" svv_status svv_build_versioned_csr(uint32_t V, uint32_t S, uint64_t n
   });
   *E_out = row_ptr[V];
   return SVV_OK;
+}
+
+extern "C" svv_status svv_build_versioned_csr(uint32_t V, uint32_t S, uint64_t n_inst, const uint32_t* src,
+                                              const uint32_t* dst, const uint32_t* w, const uint32_t* t_add,
+                                              const uint32_t* t_del, uint64_t* row_ptr, uint32_t* col,
+                                              uint32_t* weight, uint64_t* mask, uint64_t* E_out) {
+  try {
+    return build_versioned_csr(V, S, n_inst, src, dst, w, t_add, t_del, row_ptr, col, weight, mask, E_out);
+  } catch (const std::bad_alloc&) {
+    return SVV_ENOMEM;
+  }
 }
