@@ -14,7 +14,7 @@ void free_batch(svv_ctx* c) {
   p = BatchPool{};
 }
 
-// bytes one team needs for windows up to L (its share of query scratch)
+// bytes alloc_team takes, as the budget counts them
 static uint64_t team_bytes(const svv_ctx* c, uint32_t LP, uint32_t QW, uint32_t team_blocks) {
   const uint64_t V = c->g.V, E = std::max<uint32_t>(c->g.E, 1), NF = std::max<uint32_t>(c->g.NF, 1);
   const uint64_t qcap = V + E / (1u << std::min(c->solve_cs, c->relax_cs)) + 64;
@@ -75,19 +75,22 @@ svv_status ensure_pool(svv_ctx* c, int want_teams, uint32_t L) {
   const uint64_t before = c->allocated;
   int teams = want_teams;
   if (c->budget) {
-    const uint64_t per = team_bytes(c, LP, QW, total_blocks / teams + 1);
+    // a team's sums have room for any team size (fewer instances than teams)
+    const uint64_t per = team_bytes(c, LP, QW, (uint32_t)total_blocks);
     const uint64_t room = c->budget > c->allocated ? c->budget - c->allocated : 0;
-    teams = (int)std::min<uint64_t>(teams, room / (per + 4096));
+    while (teams > 0 && (uint64_t)teams * per + round256(teams * sizeof(TeamScratch)) +
+                                round256(teams * sizeof(TeamCtl) * kBatchCtl) > room)
+      --teams;
     if (teams < 1) return fail(c, SVV_ENOMEM, "batch scratch of one team exceeds the device budget");
   }
   const uint32_t team_blocks = (uint32_t)(total_blocks / teams);
   std::vector<TeamScratch> host(teams);
-  svv_status st;
-  for (int i = 0; i < teams; ++i)
-    if ((st = alloc_team(c, p.bufs, LP, QW, (uint32_t)total_blocks, host[i]))) return st;  // any team size
-  if ((st = alloc_n(c, p.bufs, (uint64_t)teams, &p.d_sc)) ||
-      (st = alloc_n(c, p.bufs, (uint64_t)teams * kBatchCtl, &p.d_ctl)))
-    return st;
+  svv_status st = SVV_OK;
+  for (int i = 0; i < teams && !st; ++i) st = alloc_team(c, p.bufs, LP, QW, (uint32_t)total_blocks, host[i]);
+  if (!st) st = alloc_n(c, p.bufs, (uint64_t)teams, &p.d_sc);
+  if (!st) st = alloc_n(c, p.bufs, (uint64_t)teams * kBatchCtl, &p.d_ctl);
+  p.bytes = c->allocated - before;  // also of a pool that stays incomplete: the next call frees it
+  if (st) return st;
   cudaError_t e = cudaMemcpy(p.d_sc, host.data(), sizeof(TeamScratch) * teams, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return cuda_fail(c, e, "uploading team scratch");
   p.want = want_teams;
@@ -95,7 +98,6 @@ svv_status ensure_pool(svv_ctx* c, int want_teams, uint32_t L) {
   p.team_blocks = team_blocks;
   p.LP = LP;
   p.QW = QW;
-  p.bytes = c->allocated - before;
   return SVV_OK;
 }
 
@@ -111,13 +113,15 @@ svv_status ensure_instances(svv_ctx* c, uint32_t n) {
   p.icap = 0;
   const uint64_t before = c->allocated;
   const uint32_t cap = std::max<uint32_t>(n, 64);
-  svv_status st;
-  if ((st = alloc_n(c, p.ibufs, cap, &p.d_inst)) || (st = alloc_n(c, p.ibufs, cap, &p.d_qerr)) ||
-      (st = alloc_n(c, p.ibufs, cap, &p.d_done)) || (st = alloc_n(c, p.ibufs, cap, &p.d_t0)) ||
-      (st = alloc_n(c, p.ibufs, cap, &p.d_t1)) || (st = alloc_n(c, p.ibufs, 1, &p.d_next)))
-    return st;
-  p.icap = cap;
+  svv_status st = alloc_n(c, p.ibufs, cap, &p.d_inst);
+  if (!st) st = alloc_n(c, p.ibufs, cap, &p.d_qerr);
+  if (!st) st = alloc_n(c, p.ibufs, cap, &p.d_done);
+  if (!st) st = alloc_n(c, p.ibufs, cap, &p.d_t0);
+  if (!st) st = alloc_n(c, p.ibufs, cap, &p.d_t1);
+  if (!st) st = alloc_n(c, p.ibufs, 1, &p.d_next);
   p.ibytes = c->allocated - before;
+  if (st) return st;
+  p.icap = cap;
   return SVV_OK;
 }
 
@@ -261,8 +265,8 @@ extern "C" svv_status svv_query_batch(svv_ctx* c, uint32_t n, svv_query_spec* sp
     c->err.clear();
     return SVV_OK;
   }
+  if ((st = ensure_instances(c, m))) return fail_all(st);  // first: the teams take what is left
   if ((st = ensure_pool(c, default_teams(c), Lmax))) return fail_all(st);
-  if ((st = ensure_instances(c, m))) return fail_all(st);
   BatchPool& p = c->batch;
   cudaError_t e = cudaMemcpyAsync(p.d_inst, inst.data(), sizeof(BatchInstance) * m, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(p.d_ctl, 0, sizeof(TeamCtl) * kBatchCtl * p.teams, s);
