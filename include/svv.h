@@ -82,6 +82,10 @@ typedef struct {
     uint32_t iters_relax;     /* frontier rounds of the multi-snapshot relaxation */
     uint32_t iters_plain_max; /* largest round count of a per-snapshot solve */
     uint32_t phase_timing;    /* 1 if the ms_* fields below were measured */
+    /* edges examined over all rounds of the two solves and of the multi-snapshot
+     * relaxation (its last slab).  A push round examines the frontier's out-edges;
+     * a pull round the in-edges (a solve counts padding slots among them) of
+     * targets that can still improve */
     uint64_t edges_relaxed_cap, edges_relaxed_cup, edges_relaxed_multi;
     /* device time of each phase (CUDA events on the query stream), when the
      * "phase_timing" tuning key is 1: intersection solve, union solve, stable

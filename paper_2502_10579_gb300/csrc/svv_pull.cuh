@@ -66,8 +66,9 @@ struct PullRound {
 // gives the value lanes in which the edge of a slot is present (kAll: every
 // edge is, and pres is not called).  Returns this lane's number of improved
 // (target, item) pairs: zero over the grid exactly when nothing changed; `key`
-// takes the best of the improved values (nf_key).  kStride: words per vertex
-// (the KL lanes of the pass are the first ones of a row).
+// takes the best of the improved values (nf_key), lane 0's `edges` the slots
+// read for targets that could still improve.  kStride: words per vertex (the KL
+// lanes of the pass are the first ones of a row).
 //
 // A target's in-edges come in the order of their weights, the best first
 // (ascending; kDesc: from the end, for widest paths).  The best that an edge
@@ -79,9 +80,9 @@ struct PullRound {
 // it - 1), so a target is done when it has been reached.
 template <class Op, int KL, int kStride, bool kAll, bool kDesc, class Pres>
 __device__ __forceinline__ uint32_t pull_items(const PullGraph& P, const PullRound& r, uint32_t gwarp, uint32_t nwarps,
-                                               unsigned lane, unsigned long long& scanned, uint32_t& key, Pres pres) {
+                                               unsigned lane, unsigned long long& edges, uint32_t& key, Pres pres) {
   constexpr int U = KL == 8 ? 2 : 4;  // edges in flight per lane
-  uint32_t changed = 0;
+  uint32_t changed = 0, seen = 0;
   for (uint32_t i = gwarp; i < P.nitems; i += nwarps) {
     const uint2 d = ld_stream(P.items + (kDesc ? P.nitems - 1u - i : i));
     const uint32_t slice = d.y >> 4, steps = (d.y & 15u) + 1u;
@@ -125,7 +126,9 @@ __device__ __forceinline__ uint32_t pull_items(const PullGraph& P, const PullRou
         if (live && s + j < steps) sw[j] = ld_stream(P.cw + slot_of(j));
       }
       live = live && gains(sw[0].y);
-      if (!__any_sync(kFullMask, live)) break;
+      const unsigned on = __ballot_sync(kFullMask, live);
+      if (!on) break;
+      seen += __popc(on) * min((uint32_t)U, steps - s);
       uint32_t pm[U];
 #pragma unroll
       for (int j = 0; j < U; ++j) {
@@ -153,7 +156,6 @@ __device__ __forceinline__ uint32_t pull_items(const PullGraph& P, const PullRou
       if (Op::kLevels && hub) live = __all_sync(kFullMask, live);
       if (!__any_sync(kFullMask, live)) break;
     }
-    if (lane == 0) scanned += 32u * min(s + (uint32_t)U, steps);
     if (hub) {
 #pragma unroll
       for (int k = 0; k < KL; ++k)
@@ -177,6 +179,7 @@ __device__ __forceinline__ uint32_t pull_items(const PullGraph& P, const PullRou
       }
     }
   }
+  if (lane == 0) edges += seen;
   return changed;
 }
 

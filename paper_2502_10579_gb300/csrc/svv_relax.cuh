@@ -37,11 +37,12 @@ __device__ __forceinline__ uint32_t relax_q(const RelaxArgs& a, bool q1, uint32_
 // At scale 20 with 533K unstable vertices and 16M subgraph edges (136 MB of
 // rows) push rounds took 270-775 us each.
 
-// the edges of one item: 32 lanes hold the steps of 32 / sp targets at a time
+// the edges of one item: 32 lanes hold the steps of 32 / sp targets at a time;
+// `edges` counts those whose source's row was read
 template <class Op, int K, bool kPart>
 __device__ __forceinline__ uint32_t relax_pull_items(const PullGraph& P, const RelaxArgs& a, bool q1, uint32_t it,
                                                      const uint32_t (&best)[K], uint32_t* s_best, unsigned gwarp,
-                                                     unsigned nwarps, unsigned lane) {
+                                                     unsigned nwarps, unsigned lane, uint32_t& edges) {
   const uint32_t lps = __ffs(a.LP) - 1;
   const uint32_t* rowmap = q1 ? a.row1 : a.row;
   const uint32_t snap = (q1 ? a.win1.b : a.win.b) + a.s0;
@@ -94,6 +95,7 @@ __device__ __forceinline__ uint32_t relax_pull_items(const PullGraph& P, const R
 #pragma unroll
           for (int kk = 0; kk < K; ++kk) gain |= Op::better(relax_q<Op>(a, q1, best[kk], w0), cur[kk]);
           if (!__any_sync(kFullMask, gain)) break;
+          edges += min((uint32_t)__popc(todo), (uint32_t)H);
           uint32_t su[H][K], ew[H];
           uint64_t e0[H], e1[H];
           bool ev[H];
@@ -150,7 +152,7 @@ template <class Op, int K>
 __device__ __noinline__ uint32_t relax_pull_round(const RelaxArgs& a, uint32_t it, StageMem* stage, unsigned gwarp,
                                                   unsigned nwarps) {
   const unsigned lane = threadIdx.x & 31u;
-  uint32_t changed = 0;
+  uint32_t changed = 0, edges = 0;
   for (int qi = 0; qi < (a.counts1 ? 2 : 1); ++qi) {
     uint32_t best[K];
 #pragma unroll
@@ -158,9 +160,12 @@ __device__ __noinline__ uint32_t relax_pull_round(const RelaxArgs& a, uint32_t i
       const uint32_t key = ld_cg(a.best + ((it % 3u) * 2u + qi) * kBestSnaps + lane + 32u * kk);
       best[kk] = Op::better(0u, 1u) ? ~key : key;
     }
-    changed += relax_pull_items<Op, K, false>(a.g.pf, a, qi != 0, it, best, stage->best[qi], gwarp, nwarps, lane);
-    changed += relax_pull_items<Op, K, true>(a.g.pp, a, qi != 0, it, best, stage->best[qi], gwarp, nwarps, lane);
+    changed += relax_pull_items<Op, K, false>(a.g.pf, a, qi != 0, it, best, stage->best[qi], gwarp, nwarps, lane,
+                                              edges);
+    changed += relax_pull_items<Op, K, true>(a.g.pp, a, qi != 0, it, best, stage->best[qi], gwarp, nwarps, lane,
+                                             edges);
   }
+  if (lane == 0 && edges) atomicAdd(&a.ctl->relaxed, (unsigned long long)edges);
   return changed;
 }
 
