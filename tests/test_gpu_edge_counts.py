@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 import oracle
+from test_gpu_pull import WEIGHTS, make_log
 from workloads.rmat import EdgeLog
 
 torch = pytest.importorskip("torch")
@@ -80,3 +81,45 @@ def test_relaxation_pulls_and_counts(svv, L, prune):
     # (16 of them), and every one of them needs at least one.
     assert counts[0] == M * D
     assert M <= counts[1] <= M * D // 2
+
+@pytest.mark.parametrize("mode", [1, 2])
+@pytest.mark.parametrize("wmax", [1, 300])
+def test_batches_on_a_graph_whose_relaxations_pull(svv, mode, wmax):
+    """The same graph in batches: teams of the one-launch kernel (with their own
+    scratch, several slabs in one launch) and query groups, every type."""
+    log = layers(2, wmax)
+    want = {t: oracle.query(log, t, 0, 0, S) for t in range(4)}
+    specs = [(t, 0, b, L) for t in range(4) for b, L in [(0, S), (S - 20, 20), (S - 40, 40), (S - 64, 64), (30, 105)]]
+    with svv.Context(0) as ctx:
+        ctx.set_tuning("batch_mode", mode)
+        ctx.set_tuning("batch_teams", 3)
+        ctx.load_log(log)
+        for _ in range(2):
+            outs, status = ctx.query_batch(specs)
+            assert status == [0] * len(specs)
+            for (t, _, b, L), out in zip(specs, outs):
+                np.testing.assert_array_equal(svv.to_u32(out), want[t][b:b + L])
+        for pair in ([(2, 0, S - 40, 40), (2, 0, S - 41, 40)], [(0, 0, S - 64, 64), (1, 0, S - 70, 64)]):
+            ctx.set_tuning("group_mix", 1)
+            outs, status = ctx.query_batch(pair)
+            for (t, _, b, L), out in zip(pair, outs):
+                np.testing.assert_array_equal(svv.to_u32(out), want[t][b:b + L])
+
+
+@pytest.mark.parametrize("kind", list(WEIGHTS))
+@pytest.mark.parametrize("V", [33, 5000])
+def test_one_launch_batches_pull_in_their_solves(svv, V, kind):
+    """The in-degrees and weights of test_gpu_pull in the one-launch kernel."""
+    log = make_log(V, WEIGHTS[kind], seed=V)
+    specs = [(t, s, b, L) for t in range(4) for s, b, L in [(0, 0, log.S), (0, 5, 40), (V - 3, 64, 6), (0, 3, 17)]]
+    want = [oracle.query(log, *q) for q in specs]
+    with svv.Context(0) as ctx:
+        ctx.set_tuning("pull_pct", 1)
+        ctx.set_tuning("batch_mode", 1)
+        ctx.load_log(log)
+        for teams in (1, 8):
+            ctx.set_tuning("batch_teams", teams)
+            outs, status = ctx.query_batch(specs)
+            assert status == [0] * len(specs)
+            for q, out, w in zip(specs, outs, want):
+                np.testing.assert_array_equal(svv.to_u32(out), w, err_msg=str(q))

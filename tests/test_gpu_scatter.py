@@ -29,3 +29,10 @@ def test_output_alignment(V):
                 got = svv.to_u32(buf)
                 np.testing.assert_array_equal(got[off:off + L * V].reshape(L, V), want[b:b + L])
                 assert (got[:off] == 0xFFFFFFF9).all() and (got[off + L * V:] == 0xFFFFFFF9).all()
+
+
+@pytest.mark.parametrize("V", [132, 256, 1020, 1024])
+def test_output_in_several_wide_tiles(V):
+    """Vertex counts that are multiples of 4: several tiles written 16 bytes at a
+    time, and a last one that is not full and goes word by word."""
+    test_output_alignment(V)
