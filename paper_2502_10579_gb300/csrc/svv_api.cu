@@ -60,7 +60,7 @@ LaunchCfg cfg_for(const svv_ctx* c, int occ, int bps) {
   int per_sm = occ;
   if (bps > 0) per_sm = std::min(per_sm, bps);
   per_sm = std::max(1, std::min(per_sm, 4));
-  return LaunchCfg{c->num_sms * per_sm, c->threads};
+  return LaunchCfg{grid_blocks(c->num_sms, per_sm), c->threads};
 }
 
 svv_status ensure_window(svv_ctx* c, uint32_t L) {

@@ -62,7 +62,7 @@ svv_status ensure_pool(svv_ctx* c, int want_teams, uint32_t L) {
   slab_shape(std::min(L, kMaxSlab), P, K);
   const uint32_t LP = P * K, QW = ceil_div(L, 64);
   const int per_sm = std::max(1, std::min(c->occ_batch, 2));
-  const int total_blocks = c->num_sms * per_sm;
+  const int total_blocks = grid_blocks(c->num_sms, per_sm);
   want_teams = std::max(1, std::min(want_teams, total_blocks));
   // the grid is split evenly, so a different team count needs a new pool
   if (p.teams && p.want == want_teams && p.LP >= LP && p.QW >= QW) return SVV_OK;

@@ -84,8 +84,8 @@ __device__ __forceinline__ unsigned ld_relaxed(const unsigned* p) {
 __device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------
-// Team barrier over `nblocks` (< 2^15) co-resident CTAs (cooperative launch),
-// with a bounded wait.  An arrival adds 1 + (add << 16) to the barrier's word
+// Team barrier over `nblocks` (<= kMaxTeamBlocks) co-resident CTAs (cooperative
+// launch), with a bounded wait.  An arrival adds 1 + (add << 16) to the barrier's word
 // with one release reduction, and every CTA polls that word until its low 16
 // bits show that all have arrived; the sum of the arrivals' `add` (the size of
 // the next round's frontier) is then in the rest of the word that was polled
@@ -106,6 +106,8 @@ struct TeamBar {
   uint32_t k;                  // barriers passed
 };
 constexpr unsigned long long kBarErr = 1ull << 52;  // error mark: above any sum of `add` (< 2^33 << 16)
+static_assert(kMaxTeamBlocks < (1u << 16), "arrivals fit the low bits");
+static_assert(kBarErr <= ~0ull / kMaxTeamBlocks, "a mark of every CTA fits above the sum");
 
 __device__ __forceinline__ bool team_sync(TeamCtl* c, uint32_t* qerr, TeamBar* tb, unsigned nblocks,
                                           unsigned long long spin_ns, uint32_t add, uint32_t& sum) {

@@ -40,6 +40,15 @@ struct alignas(128) TeamCtl {
 };
 static_assert(sizeof(TeamCtl) % 128 == 0, "TeamCtl must be cache-line sized");
 
+// CTAs of a team at most: what the barrier's word counts (team_sync)
+constexpr unsigned kMaxTeamBlocks = (1u << 12) - 1u;
+
+// a cooperative grid of per_sm CTAs per SM, within that
+inline int grid_blocks(int num_sms, int per_sm) {
+  const long long n = (long long)num_sms * per_sm;
+  return n < (long long)kMaxTeamBlocks ? (int)n : (int)kMaxTeamBlocks;
+}
+
 // In-edges for pull rounds, a lane per target (built by svv_layout.cu): slice
 // s holds the targets tgt[32 s .. 32 s + 31] (kNone: no target); an item is
 // {first row of 32 slots, slice << 4 | (steps - 1)}, and step k of it is the 32

@@ -218,7 +218,7 @@ svv_status na_setup(int dev, NaDevice** out) {
       return SVV_ECUDA;
     }
     d.base = static_cast<unsigned char*>(p);
-    d.blocks = sms * (occ < 2 ? occ : 2);
+    d.blocks = grid_blocks(sms, occ < 2 ? occ : 2);
     d.ready = true;
   }
   *out = &d;

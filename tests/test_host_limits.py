@@ -34,3 +34,11 @@ def test_layout_counters_fit_the_sums_of_a_small_device(evaluate):
     assert evaluate("kLayoutWords", [0]) == [1068]
     for n, got in zip(sms, words):
         assert got >= 1068 and got >= 32 * n, (n, got)
+
+
+def test_grids_stay_within_what_the_barrier_counts(evaluate):
+    """The error marks of 4,096 CTAs wrap the barrier's 64-bit word to no mark."""
+    sms = [1, 34, 152, 1023, 1024, 1365, 5000]
+    for per_sm in (1, 2, 3, 4):
+        for n, got in zip(sms, evaluate(f"grid_blocks((int)n, {per_sm})", sms)):
+            assert got == min(n * per_sm, 4095), (n, per_sm, got)
