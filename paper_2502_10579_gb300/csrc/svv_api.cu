@@ -486,11 +486,10 @@ static svv_status load_graph(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, con
   uint2 *d_cw, *d_nfcw;
   uint64_t* d_nfm;
   svv_status st;
-  if ((st = alloc_n(c, c->graph_bufs, (uint64_t)V + 1, &d_rp)) || (st = alloc_n(c, c->graph_bufs, V, &d_rowd)) ||
-      (st = alloc_n(c, c->graph_bufs, std::max<uint32_t>(E2, 1), &d_cw)) ||
-      (st = alloc_n(c, c->graph_bufs, (uint64_t)std::max<uint32_t>(NF, 1) * W, &d_nfm)) ||
-      (st = alloc_n(c, c->graph_bufs, std::max<uint32_t>(NF, 1), &d_nfsrc)) ||
-      (st = alloc_n(c, c->graph_bufs, std::max<uint32_t>(NF, 1), &d_nfcw))) {
+  Arrays graph;
+  graph.add((uint64_t)V + 1, &d_rp).add(V, &d_rowd).add(E2, &d_cw);
+  graph.add((uint64_t)NF * W, &d_nfm).add(NF, &d_nfsrc).add(NF, &d_nfcw);
+  if ((st = graph.alloc(c, c->graph_bufs))) {
     free_graph(c);
     return st;
   }
@@ -516,17 +515,13 @@ static svv_status load_graph(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, con
     free_graph(c);
     return fail(c, SVV_EINVAL, "graph too large for 32-bit work queues");
   }
-  if ((st = alloc_n(c, c->scratch_bufs, V, &c->rI)) || (st = alloc_n(c, c->scratch_bufs, V, &c->rU)) ||
-      (st = alloc_n(c, c->scratch_bufs, V, &c->stamp)) || (st = alloc_n(c, c->scratch_bufs, V, &c->row)) ||
-      (st = alloc_n(c, c->scratch_bufs, V, &c->uv)) || (st = alloc_n(c, c->scratch_bufs, part_words(c->num_sms), &c->part)) ||
-      (st = alloc_n(c, c->scratch_bufs, V, &c->qrow)) ||
-      (st = alloc_n(c, c->scratch_bufs, std::max<uint32_t>(E2, 1), &c->qcw)) ||
-      (st = alloc_n(c, c->scratch_bufs, std::max<uint32_t>(NF, 1), &c->qmcw)) ||
-      (st = alloc_n(c, c->scratch_bufs, qcap, &c->q0)) || (st = alloc_n(c, c->scratch_bufs, qcap, &c->q1)) ||
-      (st = alloc_n(c, c->scratch_bufs, ucap, &c->units)) ||
-      (st = alloc_n(c, c->scratch_bufs, kNumCtl, &c->ctl)) ||
-      (st = alloc_n(c, c->scratch_bufs, 6 * kBestSnaps, &c->rbest)) ||
-      (st = alloc_n(c, c->scratch_bufs, (uint64_t)V + (E2 >> 4) + 64, &c->procv))) {
+  Arrays scratch;
+  for (uint32_t** x : {&c->rI, &c->rU, &c->stamp, &c->row, &c->uv}) scratch.add(V, x);
+  scratch.add(part_words(c->num_sms), &c->part).add(V, &c->qrow);
+  scratch.add(E2, &c->qcw).add(NF, &c->qmcw);
+  scratch.add(qcap, &c->q0).add(qcap, &c->q1).add(ucap, &c->units);
+  scratch.add(kNumCtl, &c->ctl).add(6 * kBestSnaps, &c->rbest).add((uint64_t)V + (E2 >> 4) + 64, &c->procv);
+  if ((st = scratch.alloc(c, c->scratch_bufs))) {
     free_graph(c);
     return st;
   }
@@ -539,6 +534,10 @@ static svv_status load_graph(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, con
   if ((st = build_rowd(c, nfp.data(), d_rowd)) || (c->pull && (st = build_pull(c)))) {
     free_graph(c);
     return st;
+  }
+  if ((e = cudaStreamSynchronize(0)) != cudaSuccess) {  // queries may come on any stream
+    free_graph(c);
+    return cuda_fail(c, e, "loading the graph");
   }
   // out-degree over the edges present in some snapshot: a source without any
   // reaches nothing in any window (the query's result is known without a solve)

@@ -304,6 +304,29 @@ svv_status alloc_n(svv_ctx* c, std::vector<void*>& owner, uint64_t n, T** out) {
   return dev_alloc(c, owner, (size_t)n * sizeof(T), reinterpret_cast<void**>(out));
 }
 
+// Several arrays in one allocation, counted as if each had its own: cudaMalloc
+// and cudaFree of 30 arrays are a quarter of a small graph's load.
+struct Arrays {
+  std::vector<std::pair<void**, uint64_t>> list;
+  template <class T>
+  Arrays& add(uint64_t n, T** out) {
+    list.emplace_back(reinterpret_cast<void**>(out), round256(std::max<uint64_t>(n * sizeof(T), 16)));
+    return *this;
+  }
+  svv_status alloc(svv_ctx* c, std::vector<void*>& owner) {
+    uint64_t total = 0;
+    for (const auto& x : list) total += x.second;
+    void* base;
+    const svv_status st = dev_alloc(c, owner, total, &base);
+    uint64_t at = 0;
+    for (const auto& x : list) {
+      *x.first = st ? nullptr : static_cast<unsigned char*>(base) + at;
+      at += x.second;
+    }
+    return st;
+  }
+};
+
 inline uint32_t ceil_div(uint64_t a, uint64_t b) { return (uint32_t)((a + b - 1) / b); }
 
 // words of a context's per-CTA sums: 8 for each of up to 4 CTAs per SM, and on a

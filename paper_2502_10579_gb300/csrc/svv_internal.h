@@ -57,7 +57,7 @@ inline int grid_blocks(int num_sms, int per_sm) {
 constexpr uint32_t kItemSteps = 16;
 // counters of the layout builder (words); they live in the per-CTA sums of the
 // extraction, see part_words
-constexpr uint32_t kLayoutWords = 1068;
+constexpr uint32_t kLayoutWords = 2136;
 struct PullGraph {
   const uint2* items;
   const uint32_t* tgt;

@@ -32,7 +32,7 @@ constexpr uint32_t kBins = kHubDegree + 1;  // bin 0: hubs; bin 1 + kHubDegree -
 constexpr uint32_t kRankBlock = 256, kRankVerts = 1024;
 
 constexpr uint32_t kMaxSegs = kHubDegree / kItemSteps;  // items of the longest slice that is not a hub's
-constexpr uint32_t kSortBlocks = 128, kSortThreads = 1024;  // counters: 256 per block
+constexpr uint32_t kSortBlocks = 192, kSortThreads = 1024;  // of both halves; counters: 256 per block
 
 enum : int { kMetaHubs = 0, kMetaOrd = 1, kMetaRows = 2, kMetaItems = 3, kMetaMaxW = 4, kMeta = 5 };
 
@@ -42,42 +42,87 @@ struct Degrees {
   __device__ __forceinline__ uint32_t operator()(uint32_t v) const { return all[v] - (less ? less[v] : 0u); }
 };
 
+// One half of the layout under construction: the edges present in every
+// snapshot (part 0) or the partial ones (part 1).  A launch covers both, by
+// blockIdx.y: a small graph's load is a chain of launches of a few microseconds.
+struct Half {
+  Degrees deg;
+  uint32_t n, nhub, ns, nitems;  // edges, hub slices, slices, items
+  uint32_t sb;                   // blocks of a sort pass
+  uint32_t *hist, *off, *segoff;
+  unsigned long long* meta;
+  uint32_t *width, *sbase, *sitem, *start, *tgt, *counts;
+  uint2 *tpos, *items;
+  uint2* buf[2];  // the list being sorted: scratch, and the layout's own slots, which are filled afterwards
+  uint64_t* mask;
+};
+struct Halves {
+  Half h[2];
+};
+
 __device__ __forceinline__ uint32_t bin_of(uint32_t d) { return d > kHubDegree ? 0u : 1u + kHubDegree - d; }
 
-__global__ void __launch_bounds__(256) degree_kernel(const uint2* cw, uint32_t n, uint32_t* deg) {
+// exclusive prefix of x over a block of 1,024 threads, and the block's total
+__device__ __forceinline__ uint32_t block_scan(uint32_t x, uint32_t& total) {
+  __shared__ uint32_t s_w[32];
+  const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+  uint32_t incl = x;
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t a = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+    if (lane >= (unsigned)o) incl += a;
+  }
+  if (lane == 31) s_w[wid] = incl;
+  __syncthreads();
+  uint32_t base = 0;
+  total = 0;
+  for (unsigned k = 0; k < 32u; ++k) {
+    if (k < wid) base += s_w[k];
+    total += s_w[k];
+  }
+  __syncthreads();
+  return base + incl - x;
+}
+
+__global__ void __launch_bounds__(256) degree_kernel(DevGraph g, uint32_t* all, uint32_t* part) {
+  const uint2* cw = blockIdx.y ? g.nfcw : g.cw;
+  const uint32_t n = blockIdx.y ? g.NF : g.E;
+  uint32_t* deg = blockIdx.y ? part : all;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x)
     atomicAdd(deg + cw[e].x, 1u);
 }
 
-__global__ void __launch_bounds__(256) hist_kernel(Degrees deg, uint32_t V, uint32_t* hist) {
+__global__ void __launch_bounds__(256) hist_kernel(const __grid_constant__ Halves hs, uint32_t V) {
+  const Half& h = hs.h[blockIdx.y];
   __shared__ uint32_t s[kBins];
   for (uint32_t b = threadIdx.x; b < kBins; b += blockDim.x) s[b] = 0u;
   __syncthreads();
   for (size_t v = blockIdx.x * (size_t)blockDim.x + threadIdx.x; v < V; v += (size_t)gridDim.x * blockDim.x) {
-    const uint32_t d = deg((uint32_t)v);
+    const uint32_t d = h.deg((uint32_t)v);
     if (d) atomicAdd(s + bin_of(d), 1u);
   }
   __syncthreads();
   for (uint32_t b = threadIdx.x; b < kBins; b += blockDim.x)
-    if (s[b]) atomicAdd(hist + b, s[b]);
+    if (s[b]) atomicAdd(h.hist + b, s[b]);
 }
 
-// one thread: bin offsets (hubs counted apart from the sorted targets)
-__global__ void binscan_kernel(const uint32_t* hist, uint32_t* off, unsigned long long* meta) {
-  uint32_t sum = 0;
-  off[0] = 0u;
-  for (uint32_t b = 1; b < kBins; ++b) {
-    off[b] = sum;
-    sum += hist[b];
+// one CTA a half: bin offsets (hubs counted apart from the sorted targets)
+__global__ void __launch_bounds__(1024) binscan_kernel(const __grid_constant__ Halves hs) {
+  static_assert(kBins <= 1024u, "a thread per bin");
+  const Half& h = hs.h[blockIdx.y];
+  const uint32_t b = threadIdx.x;
+  uint32_t total;
+  const uint32_t at = block_scan(b && b < kBins ? h.hist[b] : 0u, total);
+  if (b < kBins) h.off[b] = at;
+  if (b == 0) {
+    h.meta[kMetaHubs] = h.hist[0];
+    h.meta[kMetaOrd] = total;
   }
-  meta[kMetaHubs] = hist[0];
-  meta[kMetaOrd] = sum;
 }
 
 // slice and lane of every target (lane 32: a hub's own slice), the targets of
 // every slice, and the slice's number of steps
-__global__ void __launch_bounds__(kRankBlock) rank_kernel(Degrees deg, uint32_t V, uint32_t nhub, uint32_t* off,
-                                                          uint2* tpos, uint32_t* tgt, uint32_t* width) {
+__global__ void __launch_bounds__(kRankBlock) rank_kernel(const __grid_constant__ Halves hs, uint32_t V) {
+  const Half& h = hs.h[blockIdx.y];
   __shared__ uint32_t s_cnt[kBins], s_base[kBins];
   const uint32_t v0 = blockIdx.x * kRankVerts;
   for (uint32_t b = threadIdx.x; b < kBins; b += blockDim.x) s_cnt[b] = 0u;
@@ -86,12 +131,12 @@ __global__ void __launch_bounds__(kRankBlock) rank_kernel(Degrees deg, uint32_t 
 #pragma unroll
   for (uint32_t j = 0; j < kRankVerts / kRankBlock; ++j) {
     const size_t v = (size_t)v0 + j * kRankBlock + threadIdx.x;
-    d[j] = v < V ? deg((uint32_t)v) : 0u;
+    d[j] = v < V ? h.deg((uint32_t)v) : 0u;
     r[j] = d[j] ? atomicAdd(s_cnt + bin_of(d[j]), 1u) : 0u;
   }
   __syncthreads();
   for (uint32_t b = threadIdx.x; b < kBins; b += blockDim.x)
-    if (s_cnt[b]) s_base[b] = atomicAdd(off + b, s_cnt[b]);
+    if (s_cnt[b]) s_base[b] = atomicAdd(h.off + b, s_cnt[b]);
   __syncthreads();
 #pragma unroll
   for (uint32_t j = 0; j < kRankVerts / kRankBlock; ++j) {
@@ -99,24 +144,24 @@ __global__ void __launch_bounds__(kRankBlock) rank_kernel(Degrees deg, uint32_t 
     const uint32_t v = v0 + j * kRankBlock + threadIdx.x;
     const uint32_t b = bin_of(d[j]), k = s_base[b] + r[j];
     if (b == 0) {
-      tpos[v] = make_uint2(k, 32u);
-      for (uint32_t l = 0; l < 32u; ++l) tgt[(size_t)k * 32u + l] = v;
-      width[k] = d[j] / 32u + (d[j] % 32u != 0u);
+      h.tpos[v] = make_uint2(k, 32u);
+      for (uint32_t l = 0; l < 32u; ++l) h.tgt[(size_t)k * 32u + l] = v;
+      h.width[k] = d[j] / 32u + (d[j] % 32u != 0u);
     } else {
-      const uint32_t slice = nhub + (k >> 5);
-      tpos[v] = make_uint2(slice, k & 31u);
-      tgt[(size_t)slice * 32u + (k & 31u)] = v;
-      atomicMax(width + slice, d[j]);
+      const uint32_t slice = h.nhub + (k >> 5);
+      h.tpos[v] = make_uint2(slice, k & 31u);
+      h.tgt[(size_t)slice * 32u + (k & 31u)] = v;
+      atomicMax(h.width + slice, d[j]);
     }
   }
 }
 
-// one CTA: exclusive scan of the slices' steps; the items of hub slices come
+// one CTA a half: exclusive scan of the slices' steps; the items of hub slices come
 // first, slice by slice, then the others by their place in the slice: segoff[j]
 // is where the items that start at step j * kItemSteps begin
-__global__ void __launch_bounds__(1024) slicescan_kernel(const uint32_t* width, uint32_t n, uint32_t nhub,
-                                                         uint32_t* sbase, uint32_t* sitem, uint32_t* segoff,
-                                                         unsigned long long* meta) {
+__global__ void __launch_bounds__(1024) slicescan_kernel(const __grid_constant__ Halves hs) {
+  const Half& h = hs.h[blockIdx.y];
+  const uint32_t n = h.ns, nhub = h.nhub;
   __shared__ uint32_t s_w[32], s_i[32], s_seg[kMaxSegs];
   const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
   if (threadIdx.x < kMaxSegs) s_seg[threadIdx.x] = 0u;
@@ -124,7 +169,7 @@ __global__ void __launch_bounds__(1024) slicescan_kernel(const uint32_t* width, 
   for (uint32_t s0 = 0; s0 < n; s0 += 1024u) {
     __syncthreads();
     const uint32_t s = s0 + threadIdx.x;
-    const uint32_t w = s < n ? width[s] : 0u, it = s < nhub ? (w + kItemSteps - 1u) / kItemSteps : 0u;
+    const uint32_t w = s < n ? h.width[s] : 0u, it = s < nhub ? (w + kItemSteps - 1u) / kItemSteps : 0u;
     if (s >= nhub)
       for (uint32_t j = 0; j * kItemSteps < w; ++j) atomicAdd(s_seg + j, 1u);
     uint32_t iw = w, ii = it;
@@ -140,41 +185,41 @@ __global__ void __launch_bounds__(1024) slicescan_kernel(const uint32_t* width, 
       cw += s_w[k], ci += s_i[k];
     }
     if (s < n) {
-      sbase[s] = bw + iw - w;
-      sitem[s] = bi + ii - it;
+      h.sbase[s] = bw + iw - w;
+      h.sitem[s] = bi + ii - it;
     }
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    meta[kMetaRows] = cw;
+    h.meta[kMetaRows] = cw;
     for (uint32_t j = 0; j < kMaxSegs; ++j) {
-      segoff[j] = ci;
+      h.segoff[j] = ci;
       ci += s_seg[j];
     }
-    meta[kMetaItems] = ci;
+    h.meta[kMetaItems] = ci;
   }
 }
 
-__global__ void __launch_bounds__(256) items_kernel(const uint32_t* width, uint32_t n, uint32_t nhub,
-                                                    const uint32_t* sbase, const uint32_t* sitem,
-                                                    const uint32_t* segoff, uint2* items) {
+__global__ void __launch_bounds__(256) items_kernel(const __grid_constant__ Halves hs) {
+  const Half& h = hs.h[blockIdx.y];
   const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const uint32_t w = width[s], b = sbase[s];
+  if (s >= h.ns) return;
+  const uint32_t w = h.width[s], b = h.sbase[s];
   for (uint32_t k = 0, j = 0; k < w; k += kItemSteps, ++j)
-    items[s < nhub ? sitem[s] + j : segoff[j] + (s - nhub)] =
+    h.items[s < h.nhub ? h.sitem[s] + j : h.segoff[j] + (s - h.nhub)] =
         make_uint2(b + k, (s << 4) | (min(w - k, kItemSteps) - 1u));
 }
 
 // every slot starts as its target's self-loop (0 where a slice has no target)
-__global__ void __launch_bounds__(256) pad_kernel(const uint2* items, uint32_t nitems, const uint32_t* tgt, uint2* cw) {
+__global__ void __launch_bounds__(256) pad_kernel(const __grid_constant__ Halves hs) {
+  const Half& h = hs.h[blockIdx.y];
   const unsigned lane = threadIdx.x & 31u;
   const size_t nw = (size_t)gridDim.x * (blockDim.x >> 5);
-  for (size_t i = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5; i < nitems; i += nw) {
-    const uint2 d = items[i];
-    const uint32_t t = tgt[(size_t)(d.y >> 4) * 32u + lane];
+  for (size_t i = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5; i < h.nitems; i += nw) {
+    const uint2 d = h.items[i];
+    const uint32_t t = h.tgt[(size_t)(d.y >> 4) * 32u + lane];
     for (uint32_t k = 0; k <= (d.y & 15u); ++k)
-      cw[(size_t)(d.x + k) * 32u + lane] = make_uint2(t == kNone ? 0u : t, 0xFFFFFFFFu);
+      h.buf[1][(size_t)(d.x + k) * 32u + lane] = make_uint2(t == kNone ? 0u : t, 0xFFFFFFFFu);
   }
 }
 
@@ -190,13 +235,15 @@ __device__ __forceinline__ uint32_t row_of(const DevGraph& g, uint32_t e) {
 }
 
 // the list to sort, {weight, edge}: the edges present in every snapshot
-// (part == 0: edge = index in the forward rows) or the partial ones (index in
+// (part 0: edge = index in the forward rows) or the partial ones (index in
 // their own list); and the largest weight
-__global__ void __launch_bounds__(256) list_kernel(DevGraph g, int part, uint2* list, unsigned long long* meta) {
-  const uint32_t n = part ? g.NF : g.E;
+__global__ void __launch_bounds__(256) list_kernel(DevGraph g, const __grid_constant__ Halves hs) {
+  const Half& h = hs.h[blockIdx.y];
+  const uint32_t n = blockIdx.y ? g.NF : g.E;
+  uint2* list = h.buf[0];
   uint32_t top = 0;
   for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
-    if (part) {
+    if (blockIdx.y) {
       const uint32_t w = g.nfcw[e].y;
       list[e] = make_uint2(w, (uint32_t)e);
       top = max(top, w);
@@ -209,66 +256,66 @@ __global__ void __launch_bounds__(256) list_kernel(DevGraph g, int part, uint2* 
     }
   }
   top = __reduce_max_sync(0xFFFFFFFFu, top);
-  if ((threadIdx.x & 31u) == 0 && top) atomicMax(meta + kMetaMaxW, (unsigned long long)top);
+  if ((threadIdx.x & 31u) == 0 && top) atomicMax(h.meta + kMetaMaxW, (unsigned long long)top);
 }
 
-__global__ void __launch_bounds__(256) rekey_kernel(DevGraph g, int part, uint2* list, uint32_t n) {
-  const uint2* cw = part ? g.nfcw : g.cw;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    list[i].x = cw[list[i].y].x;
+// the targets as keys, from buffer `from` to buffer `to` (or in place)
+__global__ void __launch_bounds__(256) rekey_kernel(DevGraph g, const __grid_constant__ Halves hs, int from, int to) {
+  const Half& h = hs.h[blockIdx.y];
+  const uint2* cw = blockIdx.y ? g.nfcw : g.cw;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < h.n; i += (size_t)gridDim.x * blockDim.x) {
+    const uint32_t e = h.buf[from][i].y;
+    h.buf[to][i] = make_uint2(cw[e].x, e);
+  }
 }
 
-// One pass of a stable radix sort by the 8 key bits at `shift`: digit counts
-// per block (blocks take consecutive ranges), their exclusive scan in digit
-// order, and the ordered move.
-__device__ __forceinline__ void sort_range(uint32_t n, uint32_t& lo, uint32_t& hi) {
-  const uint32_t per = n / gridDim.x + (n % gridDim.x != 0u);  // n may be close to 2^32
+// One pass of a stable radix sort by the 8 key bits at `shift`, from buffer
+// `from` to the other: digit counts per block (blocks take consecutive ranges),
+// their exclusive scan in digit order, and the ordered move.
+__device__ __forceinline__ void sort_range(const Half& h, uint32_t& lo, uint32_t& hi) {
+  const uint32_t n = h.n, per = n / h.sb + (n % h.sb != 0u);  // n may be close to 2^32
   lo = (uint32_t)min((unsigned long long)n, (unsigned long long)per * blockIdx.x);
   hi = (uint32_t)min((unsigned long long)n, (unsigned long long)per * blockIdx.x + per);
 }
 
-__global__ void __launch_bounds__(kSortThreads) sort_count_kernel(const uint2* in, uint32_t n, uint32_t shift,
-                                                                  uint32_t* counts) {
+__global__ void __launch_bounds__(kSortThreads) sort_count_kernel(const __grid_constant__ Halves hs, int from,
+                                                                  uint32_t shift) {
+  const Half& h = hs.h[blockIdx.y];
+  if (blockIdx.x >= h.sb) return;
+  const uint2* in = h.buf[from];
   __shared__ uint32_t s[256];
   if (threadIdx.x < 256u) s[threadIdx.x] = 0u;
   __syncthreads();
   uint32_t lo, hi;
-  sort_range(n, lo, hi);
+  sort_range(h, lo, hi);
   for (size_t i = lo + threadIdx.x; i < hi; i += kSortThreads) atomicAdd(s + ((in[i].x >> shift) & 255u), 1u);
   __syncthreads();
-  if (threadIdx.x < 256u) counts[threadIdx.x * gridDim.x + blockIdx.x] = s[threadIdx.x];
+  if (threadIdx.x < 256u) h.counts[threadIdx.x * h.sb + blockIdx.x] = s[threadIdx.x];
 }
 
-__global__ void __launch_bounds__(1024) sort_scan_kernel(uint32_t* counts, uint32_t n) {
-  __shared__ uint32_t s_w[32];
-  const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
-  uint32_t total = 0;
-  for (uint32_t i0 = 0; i0 < n; i0 += 1024u) {
-    __syncthreads();
-    const uint32_t i = i0 + threadIdx.x, c = i < n ? counts[i] : 0u;
-    uint32_t inc = c;
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t a = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-      if (lane >= (unsigned)o) inc += a;
-    }
-    if (lane == 31) s_w[wid] = inc;
-    __syncthreads();
-    uint32_t base = total;
-    for (unsigned k = 0; k < 32u; ++k) {
-      if (k < wid) base += s_w[k];
-      total += s_w[k];
-    }
-    if (i < n) counts[i] = base + inc - c;
+__global__ void __launch_bounds__(1024) sort_scan_kernel(const __grid_constant__ Halves hs) {
+  const Half& h = hs.h[blockIdx.y];
+  uint32_t base = 0;
+  for (uint32_t i0 = 0; i0 < 256u * h.sb; i0 += 1024u) {
+    const uint32_t i = i0 + threadIdx.x, n = 256u * h.sb;
+    uint32_t total;
+    const uint32_t at = block_scan(i < n ? h.counts[i] : 0u, total);
+    if (i < n) h.counts[i] = base + at;
+    base += total;
   }
 }
 
-__global__ void __launch_bounds__(kSortThreads) sort_move_kernel(const uint2* in, uint2* out, uint32_t n, uint32_t shift,
-                                                                 const uint32_t* offsets) {
+__global__ void __launch_bounds__(kSortThreads) sort_move_kernel(const __grid_constant__ Halves hs, int from,
+                                                                 uint32_t shift) {
+  const Half& h = hs.h[blockIdx.y];
+  if (blockIdx.x >= h.sb) return;
+  const uint2* in = h.buf[from];
+  uint2* out = h.buf[from ^ 1];
   __shared__ uint32_t s_base[256], s_cnt[kSortThreads / 32][256];
   const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
-  if (threadIdx.x < 256u) s_base[threadIdx.x] = offsets[threadIdx.x * gridDim.x + blockIdx.x];
+  if (threadIdx.x < 256u) s_base[threadIdx.x] = h.counts[threadIdx.x * h.sb + blockIdx.x];
   uint32_t lo, hi;
-  sort_range(n, lo, hi);
+  sort_range(h, lo, hi);
   for (size_t i0 = lo; i0 < hi; i0 += kSortThreads) {
     for (uint32_t k = lane; k < 256u; k += 32u) s_cnt[wid][k] = 0u;
     __syncwarp();
@@ -296,26 +343,27 @@ __global__ void __launch_bounds__(kSortThreads) sort_move_kernel(const uint2* in
 }
 
 // where each target's edges begin in the sorted list
-__global__ void __launch_bounds__(256) start_kernel(const uint2* list, uint32_t n, uint32_t* start) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+__global__ void __launch_bounds__(256) start_kernel(const __grid_constant__ Halves hs) {
+  const Half& h = hs.h[blockIdx.y];
+  const uint2* list = h.buf[0];
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < h.n; i += (size_t)gridDim.x * blockDim.x) {
     const uint32_t x = list[i].x;
-    if (i == 0 || list[i - 1].x != x) start[x] = (uint32_t)i;
+    if (i == 0 || list[i - 1].x != x) h.start[x] = (uint32_t)i;
   }
 }
 
-__global__ void __launch_bounds__(256) fill_kernel(DevGraph g, int part, const uint2* list, uint32_t n,
-                                                   const uint32_t* start, const uint2* tpos, const uint32_t* sbase,
-                                                   uint2* out, uint64_t* mask) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const uint2 x = list[i];  // {target, edge}
-    const uint2 tp = tpos[x.x];
-    const uint32_t k = (uint32_t)i - start[x.x], b = sbase[tp.x];
+__global__ void __launch_bounds__(256) fill_kernel(DevGraph g, const __grid_constant__ Halves hs) {
+  const Half& h = hs.h[blockIdx.y];
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < h.n; i += (size_t)gridDim.x * blockDim.x) {
+    const uint2 x = h.buf[0][i];  // {target, edge}
+    const uint2 tp = h.tpos[x.x];
+    const uint32_t k = (uint32_t)i - h.start[x.x], b = h.sbase[tp.x];
     const size_t slot = tp.y == 32u ? (size_t)b * 32u + k : (size_t)(b + k) * 32u + tp.y;
-    if (part) {
-      out[slot] = make_uint2(g.nfsrc[x.y], g.nfcw[x.y].y);
-      for (uint32_t j = 0; j < g.W; ++j) mask[slot * g.W + j] = g.nfmask[(size_t)x.y * g.W + j];
+    if (blockIdx.y) {
+      h.buf[1][slot] = make_uint2(g.nfsrc[x.y], g.nfcw[x.y].y);
+      for (uint32_t j = 0; j < g.W; ++j) h.mask[slot * g.W + j] = g.nfmask[(size_t)x.y * g.W + j];
     } else {
-      out[slot] = make_uint2(row_of(g, x.y), g.cw[x.y].y);
+      h.buf[1][slot] = make_uint2(row_of(g, x.y), g.cw[x.y].y);
     }
   }
 }
@@ -331,7 +379,8 @@ __global__ void __launch_bounds__(256) rowd_kernel(const uint32_t* rp, const uin
     rowd[v] = make_uint4(rp[v], rp[v + 1], rp[v + 1] - (nfp[v + 1] - nfp[v]), nfp[v]);
 }
 
-// row descriptors from the row offsets and the (host) prefix counts of partial edges
+// row descriptors from the row offsets and the (host) prefix counts of partial
+// edges, queued on the legacy stream
 svv_status build_rowd(svv_ctx* c, const uint32_t* nfp, uint4* rowd) {
   const uint32_t V = c->g.V;
   uint32_t* tmp = reinterpret_cast<uint32_t*>(c->q0);  // more than 2V words
@@ -340,98 +389,124 @@ svv_status build_rowd(svv_ctx* c, const uint32_t* nfp, uint4* rowd) {
     rowd_kernel<<<blocks_for(V, 1024), 256>>>(c->g.rp, tmp, V, rowd);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(0);
   return e == cudaSuccess ? SVV_OK : cuda_fail(c, e, "building the row descriptors");
 }
 
 // Build both halves of the transposed graph (edges present in every snapshot;
 // partial edges with their masks).  Runs on the legacy stream with the query
 // scratch as working memory (svv_load owns the device at that point); only
-// the layout itself is allocated.
+// the layout itself is allocated.  Two copies to the host give the sizes; one
+// launch per step for both halves, since a small graph's load is bound by the
+// chain of launches (16 vertices, 64 edges: svv_load 0.57 -> 0.33 ms; 4,096 and
+// 32,768: 0.84 -> 0.60; one allocation for many arrays is a third of that).
 svv_status build_pull(svv_ctx* c) {
   const DevGraph& g = c->g;
   const uint32_t V = g.V;
   cudaError_t e = cudaSuccess;
-  uint32_t *deg = c->stamp, *deg_p = c->rI, *start = c->rU, *width = c->row, *sbase = c->uv;
-  uint32_t* sitem = reinterpret_cast<uint32_t*>(c->q0);
-  uint2* tpos = reinterpret_cast<uint2*>(c->qrow);
-  unsigned long long* meta = reinterpret_cast<unsigned long long*>(c->part);
-  uint32_t *hist = c->part + 2 * kMeta, *off = hist + kBins;
-  uint32_t* segoff = off + kBins;
-  static_assert(2 * kMeta + 2 * kBins + kMaxSegs == kLayoutWords, "part_words");
-  uint32_t* counts = reinterpret_cast<uint32_t*>(c->ctl);  // cleared by every query
-  static_assert(sizeof(TeamCtl) * kNumCtl >= 256 * kSortBlocks * sizeof(uint32_t), "sort counters");
   auto step = [&](cudaError_t r) {
     if (e == cudaSuccess) e = r;
   };
   auto fill_words = [&](void* p, int byte, size_t n) { step(cudaMemsetAsync(p, byte, n * 4, 0)); };
+  uint32_t *deg = c->stamp, *deg_p = c->rI;
+  uint32_t *w0 = reinterpret_cast<uint32_t*>(c->q0), *w1 = reinterpret_cast<uint32_t*>(c->q1);  // more than 2V words each
+  uint2* pos = reinterpret_cast<uint2*>(c->qrow);                                               // 2V
+  unsigned long long* meta = reinterpret_cast<unsigned long long*>(c->part);
+  uint32_t* counters = c->part + 2 * 2 * kMeta;
+  static_assert(2 * (2 * kMeta + 2 * kBins + kMaxSegs) == kLayoutWords, "part_words");
+  static_assert(sizeof(TeamCtl) * kNumCtl >= 256 * kSortBlocks * sizeof(uint32_t), "sort counters");
+  Halves hs{};
+  Half &f = hs.h[0], &p = hs.h[1];
+  f.n = g.E - g.NF;
+  p.n = g.NF;
+  f.deg = Degrees{deg, deg_p};
+  p.deg = Degrees{deg_p, nullptr};
+  f.width = c->row, f.sbase = c->uv, f.sitem = w0, f.start = c->rU, f.tpos = pos;
+  p.width = w0 + V, p.sbase = w1, p.sitem = w1 + V, p.start = c->procv, p.tpos = pos + V;
+  f.buf[0] = c->qcw;
+  p.buf[0] = c->qcw + f.n;
+  for (int i = 0; i < 2; ++i) {
+    Half& h = hs.h[i];
+    h.meta = meta + i * kMeta;
+    h.hist = counters + i * (2 * kBins + kMaxSegs);
+    h.off = h.hist + kBins;
+    h.segoff = h.off + kBins;
+    // at least 1,024 edges a block, and the counters shared by the halves' sizes
+    h.sb = h.n ? std::max<uint32_t>(1, std::min<uint32_t>(ceil_div(h.n, kSortThreads),
+                                                          (uint32_t)((kSortBlocks - 1ull) * h.n / g.E)))
+               : 0u;
+  }
+  f.counts = reinterpret_cast<uint32_t*>(c->ctl);  // cleared by every query
+  p.counts = f.counts + 256 * f.sb;
+  unsigned long long m[2][kMeta] = {};
+  auto sizes = [&]() {
+    step(cudaGetLastError());
+    if (e == cudaSuccess) step(cudaMemcpy(m, meta, sizeof(m), cudaMemcpyDeviceToHost));
+    return e;
+  };
+  auto both = [](unsigned x) { return dim3(x, 2); };
   fill_words(deg, 0, V);
   fill_words(deg_p, 0, V);
-  if (g.E) degree_kernel<<<blocks_for(g.E, 1024), 256>>>(g.cw, g.E, deg);
-  if (g.NF) degree_kernel<<<blocks_for(g.NF, 1024), 256>>>(g.nfcw, g.NF, deg_p);
-  for (int part = 0; part < 2; ++part) {
-    const Degrees d{part ? deg_p : deg, part ? nullptr : deg_p};
-    const uint32_t n = part ? g.NF : g.E - g.NF;
-    PullGraph& p = part ? c->g.pp : c->g.pf;
-    unsigned long long m[kMeta] = {};
-    fill_words(c->part, 0, 2 * kMeta + 2 * kBins + kMaxSegs);
-    hist_kernel<<<blocks_for(V, 1024), 256>>>(d, V, hist);
-    binscan_kernel<<<1, 1>>>(hist, off, meta);
-    step(cudaGetLastError());
-    step(cudaMemcpy(m, meta, 2 * sizeof(m[0]), cudaMemcpyDeviceToHost));
-    if (e != cudaSuccess) return cuda_fail(c, e, "building the transposed graph");
-    const uint32_t nhub = (uint32_t)m[kMetaHubs], ns = nhub + ceil_div(m[kMetaOrd], 32);
-    uint32_t* d_tgt;
-    svv_status st = alloc_n(c, c->graph_bufs, (uint64_t)ns * 32, &d_tgt);
-    if (st) return st;
-    fill_words(d_tgt, 0xFF, (size_t)ns * 32);
-    fill_words(width, 0, std::max<uint32_t>(ns, 1));
-    rank_kernel<<<ceil_div(V, kRankVerts), kRankBlock>>>(d, V, nhub, off, tpos, d_tgt, width);
-    slicescan_kernel<<<1, 1024>>>(width, ns, nhub, sbase, sitem, segoff, meta);
-    if (n) list_kernel<<<blocks_for(part ? g.NF : g.E, 1024), 256>>>(g, part, c->qcw, meta);
-    step(cudaGetLastError());
-    step(cudaMemcpy(m, meta, sizeof(m), cudaMemcpyDeviceToHost));
-    if (e != cudaSuccess) return cuda_fail(c, e, "building the transposed graph");
-    const uint32_t nitems = (uint32_t)m[kMetaItems];
-    const uint64_t slots = m[kMetaRows] * 32;
-    uint2 *d_items, *d_cw;
-    uint64_t* d_mask = nullptr;
-    if ((st = alloc_n(c, c->graph_bufs, nitems, &d_items)) || (st = alloc_n(c, c->graph_bufs, slots, &d_cw))) return st;
-    if (part && (st = alloc_n(c, c->graph_bufs, slots * g.W, &d_mask))) return st;
-    if (n) {
-      // by weight, then by target (stable): 8 bits a pass, between the scratch
-      // edge list and the layout's own array, which is filled afterwards
-      uint2 *cur = c->qcw, *other = d_cw;
-      const unsigned sb = std::max<uint32_t>(1, std::min<uint32_t>(kSortBlocks, ceil_div(n, 4096)));
-      auto sort_by = [&](uint64_t top) {
-        for (uint32_t shift = 0; shift < 32u && (top >> shift) != 0; shift += 8u) {
-          sort_count_kernel<<<sb, kSortThreads>>>(cur, n, shift, counts);
-          sort_scan_kernel<<<1, 1024>>>(counts, 256u * sb);
-          sort_move_kernel<<<sb, kSortThreads>>>(cur, other, n, shift, counts);
-          std::swap(cur, other);
-        }
-      };
-      sort_by(m[kMetaMaxW]);
-      rekey_kernel<<<blocks_for(n, 1024), 256>>>(g, part, cur, n);
-      sort_by(V - 1u);
-      if (cur != c->qcw) step(cudaMemcpyAsync(c->qcw, cur, (size_t)n * sizeof(uint2), cudaMemcpyDeviceToDevice, 0));
-      items_kernel<<<ceil_div(ns, 256), 256>>>(width, ns, nhub, sbase, sitem, segoff, d_items);
-      pad_kernel<<<blocks_for(nitems, 8), 256>>>(d_items, nitems, d_tgt, d_cw);
-      if (part) step(cudaMemsetAsync(d_mask, 0, slots * g.W * 8, 0));
-      start_kernel<<<blocks_for(n, 1024), 256>>>(c->qcw, n, start);
-      fill_kernel<<<blocks_for(n, 256), 256>>>(g, part, c->qcw, n, start, tpos, sbase, d_cw, d_mask);
-    }
-    step(cudaGetLastError());
-    p.items = d_items;
-    p.tgt = d_tgt;
-    p.cw = d_cw;
-    p.nitems = nitems;
-    p.nhub = nhub;
-    p.slots = slots;
-    if (part) c->g.ppmask = d_mask;
+  fill_words(c->part, 0, kLayoutWords);
+  degree_kernel<<<both(blocks_for(g.E, 1024)), 256>>>(g, deg, deg_p);
+  hist_kernel<<<both(blocks_for(V, 1024)), 256>>>(hs, V);
+  binscan_kernel<<<both(1), 1024>>>(hs);
+  if (sizes() != cudaSuccess) return cuda_fail(c, e, "building the transposed graph");
+  for (int i = 0; i < 2; ++i) {
+    hs.h[i].nhub = (uint32_t)m[i][kMetaHubs];
+    hs.h[i].ns = hs.h[i].nhub + ceil_div(m[i][kMetaOrd], 32);
   }
-  step(cudaStreamSynchronize(0));
+  svv_status st;
+  uint32_t* d_tgt;
+  const uint64_t ntgt = ((uint64_t)f.ns + p.ns) * 32;
+  if ((st = alloc_n(c, c->graph_bufs, ntgt, &d_tgt))) return st;
+  f.tgt = d_tgt;
+  p.tgt = d_tgt + (uint64_t)f.ns * 32;
+  fill_words(d_tgt, 0xFF, ntgt);
+  fill_words(f.width, 0, f.ns);
+  fill_words(p.width, 0, p.ns);
+  rank_kernel<<<both(ceil_div(V, kRankVerts)), kRankBlock>>>(hs, V);
+  slicescan_kernel<<<both(1), 1024>>>(hs);
+  list_kernel<<<both(blocks_for(g.E, 1024)), 256>>>(g, hs);
+  if (sizes() != cudaSuccess) return cuda_fail(c, e, "building the transposed graph");
+  uint64_t slots[2];
+  Arrays out;
+  for (int i = 0; i < 2; ++i) {
+    hs.h[i].nitems = (uint32_t)m[i][kMetaItems];
+    slots[i] = m[i][kMetaRows] * 32;
+    out.add(hs.h[i].nitems, &hs.h[i].items).add(slots[i], &hs.h[i].buf[1]);
+  }
+  if ((st = out.add(slots[1] * g.W, &p.mask).alloc(c, c->graph_bufs))) return st;
+  if (g.E) {
+    // by weight, then by target (stable): 8 bits a pass, between the scratch
+    // list and the layout's slots, which are filled afterwards
+    const unsigned sb = std::max(f.sb, p.sb);
+    int at = 0;  // the buffer that holds the list
+    auto sort_by = [&](uint64_t top) {
+      for (uint32_t shift = 0; shift < 32u && (top >> shift) != 0; shift += 8u, at ^= 1) {
+        sort_count_kernel<<<both(sb), kSortThreads>>>(hs, at, shift);
+        sort_scan_kernel<<<both(1), 1024>>>(hs);
+        sort_move_kernel<<<both(sb), kSortThreads>>>(hs, at, shift);
+      }
+    };
+    sort_by(std::max(m[0][kMetaMaxW], m[1][kMetaMaxW]));
+    int left = 0;  // passes by target: the last one has to end in the scratch list
+    for (uint32_t shift = 0; shift < 32u && ((V - 1u) >> shift) != 0; shift += 8u) ++left;
+    rekey_kernel<<<both(blocks_for(g.E, 1024)), 256>>>(g, hs, at, left & 1);
+    at = left & 1;
+    sort_by(V - 1u);
+    items_kernel<<<both(ceil_div(std::max(f.ns, p.ns), 256)), 256>>>(hs);
+    pad_kernel<<<both(blocks_for(std::max(f.nitems, p.nitems), 8)), 256>>>(hs);
+    fill_words(p.mask, 0, slots[1] * g.W * 2);
+    start_kernel<<<both(blocks_for(g.E, 1024)), 256>>>(hs);
+    fill_kernel<<<both(blocks_for(g.E, 256)), 256>>>(g, hs);
+  }
+  step(cudaGetLastError());
   if (e != cudaSuccess) return cuda_fail(c, e, "building the transposed graph");
+  for (int i = 0; i < 2; ++i) {
+    const Half& h = hs.h[i];
+    (i ? c->g.pp : c->g.pf) = PullGraph{h.items, h.tgt, h.buf[1], h.nitems, h.nhub, slots[i]};
+  }
+  c->g.ppmask = p.mask;
   c->g.pull = 1;
   return SVV_OK;
 }

@@ -10,6 +10,7 @@ namespace svv {
 
 // threads for a loop over n items: at least 64K items each, at most 16
 inline unsigned host_threads(uint64_t n) {
+  if (n < (2u << 16)) return 1;  // asking for the number of cores takes 15-20 us
   const uint64_t hw = std::max(1u, std::thread::hardware_concurrency());
   return (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(std::min<uint64_t>(hw, 16), n >> 16));
 }

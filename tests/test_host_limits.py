@@ -27,13 +27,14 @@ def evaluate(tmp_path_factory):
 
 
 def test_layout_counters_fit_the_sums_of_a_small_device(evaluate):
-    """The layout builder keeps 1,068 words of counters in the per-CTA sums,
-    which held 32 words per SM: too few below 34 SMs."""
+    """The layout builder keeps its counters in the per-CTA sums, which held 32
+    words per SM: too few for 1,068 words below 34 SMs."""
     sms = [1, 2, 14, 17, 33, 34, 76, 152]
     words = evaluate("part_words((int)n)", sms)
-    assert evaluate("kLayoutWords", [0]) == [1068]
+    need = evaluate("kLayoutWords", [0])[0]
+    assert need >= 1068
     for n, got in zip(sms, words):
-        assert got >= 1068 and got >= 32 * n, (n, got)
+        assert got >= need and got >= 32 * n, (n, got)
 
 
 def test_grids_stay_within_what_the_barrier_counts(evaluate):
