@@ -517,8 +517,7 @@ static svv_status load_graph(svv_ctx* c, uint32_t V, uint64_t E, uint32_t S, con
   }
   Arrays scratch;
   for (uint32_t** x : {&c->rI, &c->rU, &c->stamp, &c->row, &c->uv}) scratch.add(V, x);
-  scratch.add(part_words(c->num_sms), &c->part).add(V, &c->qrow);
-  scratch.add(E2, &c->qcw).add(NF, &c->qmcw);
+  scratch.add(part_words(c->num_sms), &c->part).add((uint64_t)V + 1, &c->qrow).add(E2, &c->qcw);
   scratch.add(qcap, &c->q0).add(qcap, &c->q1).add(ucap, &c->units);
   scratch.add(kNumCtl, &c->ctl).add(6 * kBestSnaps, &c->rbest).add((uint64_t)V + (E2 >> 4) + 64, &c->procv);
   if ((st = scratch.alloc(c, c->scratch_bufs))) {
@@ -684,7 +683,6 @@ svv_status enqueue_tail(svv_ctx* c, int t, uint32_t wb, uint32_t wl, uint32_t* o
   q.cshift = c->qrs_cs;
   q.qrow = c->qrow;
   q.qcw = c->qcw;
-  q.qmcw = c->qmcw;
   q.qmask = c->qmask;
   q.ecap = c->ecap;
   q.mcap = c->mcap;
@@ -719,7 +717,6 @@ svv_status enqueue_tail(svv_ctx* c, int t, uint32_t wb, uint32_t wl, uint32_t* o
     r.uv = c->uv;
     r.qrow = c->qrow;
     r.qcw = c->qcw;
-    r.qmcw = c->qmcw;
     r.qmask = c->qmask;
     r.counts = &(c->ctl + 2)->aux[0];
     r.best = c->rbest;

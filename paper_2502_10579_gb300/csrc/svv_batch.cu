@@ -126,7 +126,6 @@ __device__ bool run_instance(const BatchArgs& b, const BatchInstance& q, uint32_
   r.cshift = b.qrs_cs;
   r.qrow = sc.qrow;
   r.qcw = sc.qcw;
-  r.qmcw = sc.qmcw;
   r.qmask = sc.qmask;
   r.ecap = sc.ecap;
   r.mcap = sc.mcap;
@@ -160,7 +159,6 @@ __device__ bool run_instance(const BatchArgs& b, const BatchInstance& q, uint32_
     x.uv = sc.uv;
     x.qrow = sc.qrow;
     x.qcw = sc.qcw;
-    x.qmcw = sc.qmcw;
     x.qmask = sc.qmask;
     x.counts = &(tc + 3)->aux[0];
     x.best = sc.rbest;

@@ -22,9 +22,9 @@ static uint64_t team_bytes(const svv_ctx* c, uint32_t LP, uint32_t QW, uint32_t 
   uint64_t b = 0;
   b += 5 * round256(V * 4);                  // rI, rU, stamp, row, uv
   b += round256(8ull * team_blocks * 4) + round256(6 * kBestSnaps * 4);  // part, rbest
-  b += round256(V * 16);                     // qrow
+  b += round256((V + 1) * 16);               // qrow
   b += round256(E * 8);                      // qcw
-  b += round256(NF * 8) + round256(NF * QW * 8);  // qmcw, qmask
+  b += round256(NF * QW * 8);                // qmask
   b += round256(V * LP * 4);                 // val
   b += 2 * round256(qcap * 8) + round256(ucap * 8);
   b += round256((V + (E >> 4) + 64) * 4);  // procv
@@ -41,8 +41,7 @@ static svv_status alloc_team(svv_ctx* c, std::vector<void*>& owner, uint32_t LP,
       (st = alloc_n(c, owner, V, &t.stamp)) || (st = alloc_n(c, owner, V, &t.row)) ||
       (st = alloc_n(c, owner, V, &t.uv)) || (st = alloc_n(c, owner, 8ull * team_blocks, &t.part)) ||
       (st = alloc_n(c, owner, 6 * kBestSnaps, &t.rbest)) ||
-      (st = alloc_n(c, owner, V, &t.qrow)) || (st = alloc_n(c, owner, E, &t.qcw)) ||
-      (st = alloc_n(c, owner, NF, &t.qmcw)) ||
+      (st = alloc_n(c, owner, V + 1, &t.qrow)) || (st = alloc_n(c, owner, E, &t.qcw)) ||
       (st = alloc_n(c, owner, NF * QW, &t.qmask)) || (st = alloc_n(c, owner, V * LP, &t.val)) ||
       (st = alloc_n(c, owner, qcap, &t.q0)) || (st = alloc_n(c, owner, qcap, &t.q1)) ||
       (st = alloc_n(c, owner, ucap, &t.units)) || (st = alloc_n(c, owner, V + (E >> 4) + 64, &t.procv)))

@@ -173,7 +173,7 @@ struct svv_ctx {
   uint32_t *rI = nullptr, *rU = nullptr, *stamp = nullptr, *row = nullptr, *uv = nullptr;
   uint32_t *part = nullptr, *qerr = nullptr, *rbest = nullptr;
   uint4* qrow = nullptr;
-  uint2 *qcw = nullptr, *qmcw = nullptr;
+  uint2* qcw = nullptr;
   unsigned long long *q0 = nullptr, *q1 = nullptr, *units = nullptr;
   uint32_t qcap = 0, ucap = 0, ecap = 0;
   svv::TeamCtl* ctl = nullptr;
@@ -190,7 +190,7 @@ struct svv_ctx {
   std::vector<void*> pair_bufs;
   uint32_t *p_uv = nullptr, *p_stamp = nullptr, *p_row1 = nullptr;
   uint4* p_qrow = nullptr;
-  uint2 *p_qcw = nullptr, *p_qmcw = nullptr;
+  uint2* p_qcw = nullptr;
   uint64_t* p_qmask = nullptr;
   uint32_t* p_val = nullptr;
   unsigned long long *p_q0 = nullptr, *p_q1 = nullptr, *p_units = nullptr;

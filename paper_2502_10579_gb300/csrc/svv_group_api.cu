@@ -163,7 +163,7 @@ void free_pair(svv_ctx* c) {
   c->pair_bufs.clear();
   c->p_uv = c->p_stamp = c->p_row1 = nullptr;
   c->p_qrow = nullptr;
-  c->p_qcw = c->p_qmcw = nullptr;
+  c->p_qcw = nullptr;
   c->p_qmask = nullptr;
   c->p_val = nullptr;
   c->p_q0 = c->p_q1 = c->p_units = nullptr;
@@ -179,9 +179,8 @@ svv_status ensure_pair_rows(svv_ctx* c, uint32_t LP) {
   // every array holds two queries' worth of what the single-query scratch holds
   svv_status st;
   if ((st = alloc_n(c, c->pair_bufs, 2 * V, &c->p_uv)) || (st = alloc_n(c, c->pair_bufs, 2 * V, &c->p_stamp)) ||
-      (st = alloc_n(c, c->pair_bufs, V, &c->p_row1)) || (st = alloc_n(c, c->pair_bufs, 2 * V, &c->p_qrow)) ||
+      (st = alloc_n(c, c->pair_bufs, V, &c->p_row1)) || (st = alloc_n(c, c->pair_bufs, 2 * V + 1, &c->p_qrow)) ||
       (st = alloc_n(c, c->pair_bufs, 2 * (uint64_t)c->ecap, &c->p_qcw)) ||
-      (st = alloc_n(c, c->pair_bufs, 2 * (uint64_t)std::max<uint32_t>(c->g.NF, 1), &c->p_qmcw)) ||
       (st = alloc_n(c, c->pair_bufs, 2 * c->mcap, &c->p_qmask)) ||
       (st = alloc_n(c, c->pair_bufs, need_v, &c->p_val)) ||
       (st = alloc_n(c, c->pair_bufs, 2 * (uint64_t)c->ucap, &c->p_units)) ||
@@ -239,7 +238,6 @@ svv_status enqueue_pair_tail(svv_ctx* c, const BatchInstance* inst, uint32_t* co
   q.cshift = c->qrs_cs;
   q.qrow = c->p_qrow;
   q.qcw = c->p_qcw;
-  q.qmcw = c->p_qmcw;
   q.qmask = c->p_qmask;
   q.ecap = (uint32_t)std::min<uint64_t>(2 * (uint64_t)c->ecap, 0xFFFFFFFFull);
   q.mcap = c->p_mcap;  // what the pair mask array holds
@@ -266,7 +264,6 @@ svv_status enqueue_pair_tail(svv_ctx* c, const BatchInstance* inst, uint32_t* co
   r.uv = c->p_uv;
   r.qrow = c->p_qrow;
   r.qcw = c->p_qcw;
-  r.qmcw = c->p_qmcw;
   r.qmask = c->p_qmask;
   r.counts = &(c->ctl + 2)->aux[0];
   r.counts1 = &(c->ctl + 6)->aux[0];

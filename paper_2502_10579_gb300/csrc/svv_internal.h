@@ -145,10 +145,13 @@ struct QrsArgs {
   unsigned long long* units;  // row | chunk << 32 over unstable rows
   uint32_t ucap;
   uint32_t cshift;
-  uint4* qrow;            // [V] per row: {first all-window edge, first other edge, how many of each}
-  uint2* qcw;             // [E] all-window edges (target row, weight): room for all out-edges of every row
-  uint2* qmcw;            // [NF] the others
-  uint64_t* qmask;        // [NF*QW] their window-rebased masks
+  // [V + 1] per row: {where its room in qcw begins, its first mask, number of
+  // all-window edges, number of others}; the entry after the last row ends its room
+  uint4* qrow;
+  // [E] (target row, weight): a row has room for all its out-edges, the all-window
+  // ones from the front, the others from the back
+  uint2* qcw;
+  uint64_t* qmask;        // [NF*QW] window-rebased masks of the others, from the front
   uint32_t ecap;
   unsigned long long mcap;  // words
   TeamCtl* ctl;           // aux[0]=U, aux[1]=#units, aux[2]=E_Q, aux[3]=#masked
@@ -177,7 +180,6 @@ struct RelaxArgs {
   const uint32_t* uv;
   const uint4* qrow;
   const uint2* qcw;
-  const uint2* qmcw;
   const uint64_t* qmask;
   const unsigned int* counts;  // qrs team aux: [0]=U
   // a second query relaxed in the same launch (counts1 null: none): its rows
@@ -260,7 +262,7 @@ struct BatchInstance {
 struct TeamScratch {
   uint32_t *rI, *rU, *stamp, *row, *uv, *part, *rbest;
   uint4* qrow;
-  uint2 *qcw, *qmcw;
+  uint2* qcw;
   uint64_t* qmask;
   uint32_t* val;
   unsigned long long *q0, *q1, *units;

@@ -11,14 +11,14 @@
 // relaxation (which reads the addition edges directly).  The kept edges are
 // those whose source and target are both unstable and that are present in at
 // least one window snapshot; per row, edges present in every window snapshot
-// come first (Section 4.1), followed by the rest with masks rebased so that bit
-// i is snapshot win_begin+i.
+// come first (Section 4.1).  The rest, with masks rebased so that bit i is
+// snapshot win_begin+i, fill the row's room from its end.
 //
 // One cooperative launch, three phases separated by the team barrier:
 //   P1 per-CTA counts of unstable vertices, their work units and out-edges;
 //   P2 rows in vertex order (CTA offsets from P1), row -> vertex map, units,
 //      and each row's place in the edge arrays, with room for all its out-edges;
-//   P3 fill: the kept edges of every unit behind those its row already holds.
+//   P3 fill: the kept edges of every unit next to those its row already holds.
 // The edges are walked once.  Counting the kept edges first, to pack the rows,
 // walked them twice, at one CTA per SM (114 registers): 121 us instead of 79 at
 // scale 20 with 111K unstable vertices, 458 instead of 311 with 533K.  Two CTAs

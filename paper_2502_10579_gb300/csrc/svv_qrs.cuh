@@ -69,7 +69,7 @@ __device__ __forceinline__ uint32_t unstable4(const QrsArgs& a, const uint32_t* 
 
 // Walk the edges of every unit in the queue (warp-balanced, as in the solve),
 // classify each edge as all-window (F) or masked (M) kept edge, and write the
-// kept ones behind those their rows already hold.  Returns (in lane 0) the
+// kept ones next to those their rows already hold.  Returns (in lane 0) the
 // numbers of kept and of masked edges.  With a second query (a.rI1), rows from
 // U0 on are that query's: its edges are classified against its own row map and
 // window.
@@ -149,22 +149,25 @@ __device__ __forceinline__ uint2 qrs_fill(const QrsArgs& a, const Team& t, uint3
         const unsigned bF = __ballot_sync(kFullMask, isF[h]), bM = __ballot_sync(kFullMask, isM[h]);
         const int leader = __ffs(grp) - 1;
         const uint32_t nF = __popc(grp & bF), nM = __popc(grp & bM);
-        uint32_t baseF = 0, baseM = 0;
         uint4* d = a.qrow + rk;
-        uint2 at = make_uint2(0u, 0u);
+        uint32_t baseF = 0, baseM = 0, baseE = 0;  // baseE: where the row's masked edges go on, downwards
         if (lane == (unsigned)leader && p < total && (nF || nM)) {
-          at = __ldcg(reinterpret_cast<const uint2*>(d));  // {first full edge, first masked edge}
-          if (nF) baseF = atomicAdd(&d->z, nF);
-          if (nM) baseM = atomicAdd(&d->w, nM);
+          const uint2 at = __ldcg(reinterpret_cast<const uint2*>(d));  // {first slot, first mask}
+          const uint32_t end = __ldcg(&d[1].x);
+          const uint32_t oF = nF ? atomicAdd(&d->z, nF) : 0u, oM = nM ? atomicAdd(&d->w, nM) : 0u;
+          baseF = at.x + oF;
+          baseM = at.y + oM;
+          baseE = end - 1u - oM;
         }
-        baseF = __shfl_sync(kFullMask, at.x + baseF, leader);
-        baseM = __shfl_sync(kFullMask, at.y + baseM, leader);
+        baseF = __shfl_sync(kFullMask, baseF, leader);
+        baseM = __shfl_sync(kFullMask, baseM, leader);
+        baseE = __shfl_sync(kFullMask, baseE, leader);
         if (isF[h]) {
           a.qcw[baseF + __popc(grp & bF & lt)] = make_uint2(rx[h], w[h]);
         } else if (isM[h]) {
-          const uint32_t pos = baseM + __popc(grp & bM & lt);
-          a.qmcw[pos] = make_uint2(rx[h], w[h]);
-          uint64_t* out = a.qmask + (size_t)pos * a.QW;
+          const uint32_t k = __popc(grp & bM & lt);
+          a.qcw[baseE - k] = make_uint2(rx[h], w[h]);
+          uint64_t* out = a.qmask + (size_t)(baseM + k) * a.QW;
           const uint32_t wb = (a.rI1 && rk >= U0) ? a.win1.b : a.win.b;
           for (uint32_t j = 0; j < a.QW; ++j) {
             uint64_t word = mask_extract(g.nfmask + (size_t)mi[h] * g.W, g.W, wb + 64u * j);
@@ -292,6 +295,7 @@ __device__ inline bool qrs_team(const QrsArgs& a, const Team& t) {
       }
     }
   }
+  if (b == 0 && tid == 0) a.qrow[base.rows] = make_uint4(base.deg, base.part, 0u, 0u);
   if (!t.sync()) return false;
 
   // ---- P3: fill

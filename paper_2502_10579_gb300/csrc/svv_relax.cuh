@@ -208,6 +208,7 @@ __device__ __noinline__ RelaxDone relax_push_round(const RelaxArgs& a, const Rel
     const uint32_t ui = t0 + grp;
     uint32_t beg = 0, end = 0;  // of the unit, counted over the row's all-window edges and then the others
     uint4 d = make_uint4(0u, 0u, 0u, 0u);
+    uint32_t room_end = 0;
     bool q1 = false;  // the unit's row belongs to the second query
     uint32_t sv[K];
 #pragma unroll
@@ -217,6 +218,7 @@ __device__ __noinline__ RelaxDone relax_push_round(const RelaxArgs& a, const Rel
       const uint32_t r = (uint32_t)u, ch = (uint32_t)(u >> 32);
       q1 = r >= U0;
       d = a.qrow[r];
+      room_end = a.qrow[r + 1].x;
       beg = ch << a.cshift;
       end = min(d.z + d.w, beg + (1u << a.cshift));
       const uint32_t* src = a.val + ((size_t)r << lps) + gl;
@@ -234,12 +236,12 @@ __device__ __noinline__ RelaxDone relax_push_round(const RelaxArgs& a, const Rel
       for (int k = 0; k < NW; ++k) mw[k] = slab[k];
       if (e < end) {
         const bool full = e < d.z;
-        const uint32_t k = full ? d.x + e : d.y + (e - d.z);
-        const uint2 ew = (full ? a.qcw : a.qmcw)[k];
+        const uint32_t m = e - d.z;  // of the others, which end the row's room
+        const uint2 ew = a.qcw[full ? d.x + e : room_end - 1u - m];
         xr = ew.x;
         w = ew.y;
         if (!full) {
-          const uint64_t* mp = a.qmask + (size_t)k * a.QW;
+          const uint64_t* mp = a.qmask + (size_t)(d.y + m) * a.QW;
 #pragma unroll
           for (int k = 0; k < NW; k += 2) {
             const uint64_t x = mask_extract(mp, a.QW, a.s0 + 32u * k);
