@@ -45,12 +45,6 @@ __device__ __forceinline__ uint2 ld_row_span(const DevGraph& g, uint32_t v) {
   return __ldg(reinterpret_cast<const uint2*>(g.rowd + v));
 }
 
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
 __device__ __forceinline__ unsigned long long global_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

@@ -46,7 +46,10 @@ __global__ void __launch_bounds__(256) group_lanes_kernel(LanesArgs a) {
   }
 }
 
-// two-lane groups fit 40 registers: 3 CTAs per SM, as the single solve
+// two-lane groups at 3 CTAs per SM (40 registers), as the single solve; the
+// choice is from the older pull loop, which fitted: now 4 to 112 bytes of spill
+// stores, 120 in the mixed pair.  Four and eight lanes have 64 registers and
+// spill only in the mixed union solve of eight (92 bytes).
 template <class Op, int KL, int PRED>
 __global__ void __launch_bounds__(kGroupThreads, KL == 2 ? 3 : 2) group_solve_kernel(GroupArgs a) {
   __shared__ StageMem s_stage;

@@ -183,7 +183,7 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, StageMem* st
   fold_keys();
   uint32_t queued = stage_flush_cta(st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
   publish_keys(1u);
-  uint32_t n = 0;  // the round's frontier: units, or vertices after a pull round
+  uint32_t n = 0;  // the round's frontier: units, or improved (target, item) pairs after a pull round
   bool dense = false;
   if (!t.sync(queued, n)) return false;
 
@@ -200,8 +200,9 @@ __device__ bool group_solve_team(const GroupArgs& a, const Team& t, StageMem* st
     }
     n = min(n, a.qcap);
     // After a push round the frontier is a unit queue of n units; after a
-    // pull round it is the n vertices stamped with `it`.  A large frontier is
-    // pulled, a small one pushed.
+    // pull round it is the vertices stamped with `it` (n counts as in the
+    // single solve, once per pass).  A large frontier is pulled, a small one
+    // pushed.
     const bool can_pull = g.pull != 0u && a.pull_units != 0u;
     const bool pull = can_pull && (dense ? (n > a.push_verts) : (n > a.pull_units));
     if (gtid == 0) {

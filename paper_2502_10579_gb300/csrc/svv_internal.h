@@ -123,8 +123,8 @@ struct SolveArgs {
   uint32_t pcap;
   // direction switch (needs the transposed graph): a round whose frontier
   // holds more than pull_units units runs as a pull pass over every vertex's
-  // in-edges; after a pull round that changed more than push_verts vertices the
-  // next round pulls again.  0 disables pulling.
+  // in-edges; after a pull round with more than push_verts improved (target,
+  // item) pairs the next round pulls again.  0 disables pulling.
   uint32_t pull_units, push_verts;
   // test hook (0 = off): CTA skip_arrival-1 leaves before its first barrier
   // arrival, so the other CTAs' bounded waits expire (SVV_ETIMEOUT)
@@ -157,7 +157,7 @@ struct QrsArgs {
   TeamCtl* ctl;           // aux[0]=U, aux[1]=#units, aux[2]=E_Q, aux[3]=#masked
   uint32_t* qerr;
   unsigned long long spin_ns;
-  unsigned long long* trace;  // optional: start ns of each of the five passes, then the end
+  unsigned long long* trace;  // optional: start ns of the three phases (the third in [2], [3] and [4]), then the end
   uint32_t rowcap;        // rows the row arrays hold (uv, qrow)
   // a second query extracted in the same launch (rI1 null: none), same window
   // length: its rows, units, edges and masks follow the first query's; its

@@ -170,7 +170,8 @@ __device__ __noinline__ uint32_t relax_pull_round(const RelaxArgs& a, uint32_t i
 }
 
 // One push round (Algorithm 2 over the frontier's units) and its flush.  Out of
-// line, so that the loop has the registers to itself; kNote: also keep the best
+// line, so that the loop has the registers to itself (64; rows of 32 to 128
+// values store 16 to 96 bytes of them on the stack all the same); kNote: also keep the best
 // improved value of every snapshot, for the bound of a pull round that follows.
 struct RelaxRound {
   uint32_t n, it, U0, gwarp, nwarps;
@@ -338,7 +339,9 @@ __device__ bool relax_team(const RelaxArgs& a, const Team& t, StageMem* stage) {
   // A pull round looks at every in-edge of the unstable vertices (about U * E /
   // V), a push round at the frontier's share of the kept edges: pull when that
   // is more than 0.4 of the former (measured at 0.35-0.41: 308 us against 271,
-  // 438 against 412; at 0.5: 531 against 579, at 0.7: 525 against 775).
+  // 438 against 412; at 0.5: 531 against 579, at 0.7: 525 against 775; rounds of
+  // one scale-20 query with 533K unstable vertices).  Where the unstable vertices'
+  // mean in-degree is above E / V a pull costs more than this counts.
   // pull_above is that frontier in units; most queries never get there.
   const uint32_t all_units = U + (a.counts[2] >> a.cshift);
   const float few = 0.4f * (float)U * ((float)g.E / (float)g.V), kept = (float)a.counts[2];
@@ -481,7 +484,7 @@ __device__ bool relax_team(const RelaxArgs& a, const Team& t, StageMem* stage) {
   }
   uint32_t queued = stage_flush_cta(st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
   publish_best(1u);
-  uint32_t n = 0;  // the round's frontier: units, or rows after a pull round
+  uint32_t n = 0;  // the round's frontier: units, or improved (row, item part) pairs after a pull round
   bool dense = false;
   if (!t.sync(queued, n)) return false;
 
@@ -497,7 +500,8 @@ __device__ bool relax_team(const RelaxArgs& a, const Team& t, StageMem* stage) {
       break;
     }
     n = min(n, a.qcap);
-    // after a pull round n counts rows: an average row has all_units / U units
+    // after a pull round n counts a row once for every part of an item that
+    // improved it; taken as a row, which has all_units / U units on average
     const bool pull = may_pull && (dense ? (float)n * ((float)all_units / (float)U) : (float)n) > (float)pull_above;
     if (gtid == 0) {
       atomicExch(&c->qn[clr], 0u);

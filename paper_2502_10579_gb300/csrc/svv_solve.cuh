@@ -102,7 +102,7 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, StageMem* stage) {
   fold_key();
   uint32_t queued = stage_flush_cta(st, a.q1, &c->qn[1], a.qcap, c, a.qerr, lane);
   publish_key(&c->aux[1]);
-  uint32_t n = 0;  // the round's frontier: units, or vertices after a pull round
+  uint32_t n = 0;  // the round's frontier: units, or improved (target, item) pairs after a pull round
   bool dense = false;
   if (!t.sync(queued, n)) return false;
 
@@ -119,9 +119,11 @@ __device__ bool solve_team(const SolveArgs& a, const Team& t, StageMem* stage) {
     }
     n = min(n, a.qcap);
     // How this round runs.  After a push round the frontier is a unit queue of
-    // n units; after a pull round it is the n vertices stamped with `it`.  A
-    // large frontier is pulled: every vertex takes the best candidate over
-    // its in-edges (no queue, one atomic per chunk); a small one is pushed.
+    // n units; after a pull round it is the vertices stamped with `it`, and n
+    // counts a vertex once, a hub once per item that improved it (so hubs keep
+    // pulling a little longer).  A large frontier is pulled: every vertex takes
+    // the best candidate over its in-edges (no queue, one reduction per target
+    // and item); a small one is pushed.
     const bool can_pull = g.pull != 0u && a.pull_units != 0u;
     const bool pull = can_pull && (dense ? (n > a.push_verts) : (n > a.pull_units));
     if (gtid == 0) {
