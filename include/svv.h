@@ -210,6 +210,8 @@ svv_status svv_query_batch(svv_ctx *ctx, uint32_t n, svv_query_spec *specs, void
  * leaves); a request that does not fit is refused with SVV_EBUSY until earlier
  * results are released -- that is the admission control.  The kernel leaves
  * after an idle period and is relaunched by the next svv_submit or svv_poll.
+ * svv_query_batch in one launch runs on the same teams, after the requests
+ * already submitted.
  * That is the mode below 2M vertices.  From 2M vertices ("batch_mode" as set
  * when the server starts: 0 = by graph size, 1 = live kernel, 2 = groups),
  * where one request already fills the GPU, requests run in QUERY GROUPS

@@ -265,8 +265,15 @@ extern "C" svv_status svv_query_batch(svv_ctx* c, uint32_t n, svv_query_spec* sp
     return SVV_OK;
   }
   if ((st = ensure_instances(c, m))) return fail_all(st);  // first: the teams take what is left
-  if ((st = ensure_pool(c, default_teams(c), Lmax))) return fail_all(st);
   BatchPool& p = c->batch;
+  const bool live = serving_live(c);
+  if (live && (st = quiesce_live(c))) return fail_all(st);
+  const int served = p.want;  // the server's teams, and its longest window
+  const uint32_t Ls = live ? c->serve.maxL : 0u;
+  if ((st = ensure_pool(c, default_teams(c), std::max(Lmax, Ls)))) {
+    if (live && !p.teams) ensure_pool(c, served, Ls);  // what it had
+    return fail_all(st);
+  }
   cudaError_t e = cudaMemcpyAsync(p.d_inst, inst.data(), sizeof(BatchInstance) * m, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(p.d_ctl, 0, sizeof(TeamCtl) * kBatchCtl * p.teams, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(p.d_next, 0, sizeof(unsigned), s);

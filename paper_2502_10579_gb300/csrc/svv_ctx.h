@@ -407,6 +407,10 @@ svv_status status_of(uint32_t qerr, uint32_t done);
 svv_status check_spec(const svv_ctx* c, const svv_query_spec& q);
 bool batch_one_launch(const svv_ctx* c);
 svv_status reserve_window(svv_ctx* c, uint32_t L);
+// A live server runs on the batch teams' scratch and barriers: let it finish what
+// was submitted and leave (the next svv_submit or svv_poll launches it again).
+bool serving_live(const svv_ctx* c);
+svv_status quiesce_live(svv_ctx* c);
 
 // While an in-order server is active it shares the single-query scratch: a
 // call that uses that scratch on another stream is ordered after the requests

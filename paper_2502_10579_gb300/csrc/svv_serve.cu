@@ -317,6 +317,21 @@ ServeSlot* slot_of(svv_ctx* c, uint64_t ticket) {
 }
 
 }  // namespace
+
+bool serving_live(const svv_ctx* c) { return c->serve.active && !c->serve.in_order; }
+
+svv_status quiesce_live(svv_ctx* c) {
+  ServeState& v = c->serve;
+  volatile uint32_t* stop = reinterpret_cast<volatile uint32_t*>(v.h_ctrl) + 1;
+  svv_status st = ensure_running(c);  // requests left waiting by a kernel that went idle
+  if (st) return st;
+  *stop = 1u;  // looked at when no request waits
+  std::atomic_thread_fence(std::memory_order_seq_cst);
+  const cudaError_t e = cudaStreamSynchronize(v.stream);
+  *stop = 0u;
+  return e == cudaSuccess ? SVV_OK : cuda_fail(c, e, "serving kernel");
+}
+
 }  // namespace svv
 
 using namespace svv;
