@@ -29,7 +29,7 @@ void free_graph(svv_ctx* c) {
   if (c->copy_stream) cudaStreamSynchronize(c->copy_stream);
   free_list(c, c->bstage_bufs);
   c->bstage[0] = c->bstage[1] = nullptr;
-  c->bstage_cap = 0;
+  c->bstage_cap = c->bstage_bytes = 0;
   c->allocated = 0;
   c->loaded = false;
   c->g = DevGraph{};
@@ -858,12 +858,14 @@ static svv_status ensure_bstage(svv_ctx* c, uint64_t words) {
   if (words <= c->bstage_cap) return SVV_OK;
   cudaStreamSynchronize(c->copy_stream);
   free_list(c, c->bstage_bufs);
-  c->allocated -= std::min<uint64_t>(c->allocated, 2 * round256(c->bstage_cap * 4));
+  c->allocated -= std::min(c->allocated, c->bstage_bytes);
   c->bstage[0] = c->bstage[1] = nullptr;
   c->bstage_cap = 0;
-  svv_status st;
-  if ((st = alloc_n(c, c->bstage_bufs, words, &c->bstage[0])) || (st = alloc_n(c, c->bstage_bufs, words, &c->bstage[1])))
-    return st;
+  const uint64_t before = c->allocated;
+  svv_status st = alloc_n(c, c->bstage_bufs, words, &c->bstage[0]);
+  if (!st) st = alloc_n(c, c->bstage_bufs, words, &c->bstage[1]);
+  c->bstage_bytes = c->allocated - before;
+  if (st) return st;
   c->bstage_cap = words;
   return SVV_OK;
 }

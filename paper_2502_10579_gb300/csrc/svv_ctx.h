@@ -188,6 +188,7 @@ struct svv_ctx {
   // a two-query group's tails in one relaxation launch: both queries' rows,
   // subgraph edges and masks in one set of arrays (allocated on first use)
   std::vector<void*> pair_bufs;
+  uint64_t pair_bytes = 0;  // of pair_bufs, as counted in `allocated`
   uint32_t *p_uv = nullptr, *p_stamp = nullptr, *p_row1 = nullptr;
   uint4* p_qrow = nullptr;
   uint2* p_qcw = nullptr;
@@ -200,6 +201,7 @@ struct svv_ctx {
   uint32_t* bstage[2] = {nullptr, nullptr};
   uint64_t bstage_cap = 0;      // words per slot
   std::vector<void*> bstage_bufs;
+  uint64_t bstage_bytes = 0;
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t ev_done[2] = {}, ev_copied[2] = {};
 
@@ -242,6 +244,7 @@ struct svv_ctx {
   int occ_group2 = 0;  // of 2 lanes
   bool group_ready = false;
   std::vector<void*> group_bufs;
+  uint64_t group_bytes = 0;
   uint32_t *gcap = nullptr, *gcup = nullptr, *gnfl = nullptr, *gipl = nullptr, *gerr = nullptr;
   uint32_t* gI[svv::kGroupMax] = {};
   uint32_t* gU[svv::kGroupMax] = {};

@@ -12,6 +12,8 @@ void free_group(svv_ctx* c) {
   c->last_rI = c->last_rU = c->last_row = nullptr;
   for (void* p : c->group_bufs) cudaFree(p);
   c->group_bufs.clear();
+  c->allocated -= std::min(c->allocated, c->group_bytes);
+  c->group_bytes = 0;
   c->gcap = c->gcup = c->gnfl = c->gipl = c->gerr = nullptr;
   for (int k = 0; k < kGroupMax; ++k) c->gI[k] = c->gU[k] = nullptr;
   c->group_ready = false;
@@ -20,18 +22,18 @@ void free_group(svv_ctx* c) {
 svv_status ensure_group(svv_ctx* c) {
   if (c->group_ready) return SVV_OK;
   const uint64_t V = c->g.V, NF = std::max<uint32_t>(c->g.NF, 1);
-  svv_status st;
-  if ((st = alloc_n(c, c->group_bufs, V * kGroupMax, &c->gcap)) ||
-      (st = alloc_n(c, c->group_bufs, V * kGroupMax, &c->gcup)) || (st = alloc_n(c, c->group_bufs, NF, &c->gnfl)) ||
-      (st = alloc_n(c, c->group_bufs, std::max<uint64_t>(c->g.pp.slots, 1), &c->gipl)) || (st = alloc_n(c, c->group_bufs, 1, &c->gerr))) {
+  const uint64_t before = c->allocated;
+  svv_status st = alloc_n(c, c->group_bufs, V * kGroupMax, &c->gcap);
+  if (!st) st = alloc_n(c, c->group_bufs, V * kGroupMax, &c->gcup);
+  if (!st) st = alloc_n(c, c->group_bufs, NF, &c->gnfl);
+  if (!st) st = alloc_n(c, c->group_bufs, std::max<uint64_t>(c->g.pp.slots, 1), &c->gipl);
+  if (!st) st = alloc_n(c, c->group_bufs, 1, &c->gerr);
+  for (int k = 0; k < kGroupMax && !st; ++k)
+    if (!(st = alloc_n(c, c->group_bufs, V, &c->gI[k]))) st = alloc_n(c, c->group_bufs, V, &c->gU[k]);
+  c->group_bytes = c->allocated - before;
+  if (st) {
     free_group(c);
     return st;
-  }
-  for (int k = 0; k < kGroupMax; ++k) {
-    if ((st = alloc_n(c, c->group_bufs, V, &c->gI[k])) || (st = alloc_n(c, c->group_bufs, V, &c->gU[k]))) {
-      free_group(c);
-      return st;
-    }
   }
   c->group_ready = true;
   return SVV_OK;
@@ -161,6 +163,8 @@ void free_pair(svv_ctx* c) {
   if (c->p_row1 && c->last_row == c->p_row1) c->last_row = nullptr;
   for (void* p : c->pair_bufs) cudaFree(p);
   c->pair_bufs.clear();
+  c->allocated -= std::min(c->allocated, c->pair_bytes);
+  c->pair_bytes = 0;
   c->p_uv = c->p_stamp = c->p_row1 = nullptr;
   c->p_qrow = nullptr;
   c->p_qcw = nullptr;
@@ -177,15 +181,19 @@ svv_status ensure_pair_rows(svv_ctx* c, uint32_t LP) {
   if (c->p_uv && need_v <= c->p_valcap && 2 * c->mcap <= c->p_mcap) return SVV_OK;
   free_pair(c);
   // every array holds two queries' worth of what the single-query scratch holds
-  svv_status st;
-  if ((st = alloc_n(c, c->pair_bufs, 2 * V, &c->p_uv)) || (st = alloc_n(c, c->pair_bufs, 2 * V, &c->p_stamp)) ||
-      (st = alloc_n(c, c->pair_bufs, V, &c->p_row1)) || (st = alloc_n(c, c->pair_bufs, 2 * V + 1, &c->p_qrow)) ||
-      (st = alloc_n(c, c->pair_bufs, 2 * (uint64_t)c->ecap, &c->p_qcw)) ||
-      (st = alloc_n(c, c->pair_bufs, 2 * c->mcap, &c->p_qmask)) ||
-      (st = alloc_n(c, c->pair_bufs, need_v, &c->p_val)) ||
-      (st = alloc_n(c, c->pair_bufs, 2 * (uint64_t)c->ucap, &c->p_units)) ||
-      (st = alloc_n(c, c->pair_bufs, 2 * (uint64_t)c->qcap, &c->p_q0)) ||
-      (st = alloc_n(c, c->pair_bufs, 2 * (uint64_t)c->qcap, &c->p_q1))) {
+  const uint64_t before = c->allocated;
+  svv_status st = alloc_n(c, c->pair_bufs, 2 * V, &c->p_uv);
+  if (!st) st = alloc_n(c, c->pair_bufs, 2 * V, &c->p_stamp);
+  if (!st) st = alloc_n(c, c->pair_bufs, V, &c->p_row1);
+  if (!st) st = alloc_n(c, c->pair_bufs, 2 * V + 1, &c->p_qrow);
+  if (!st) st = alloc_n(c, c->pair_bufs, 2 * (uint64_t)c->ecap, &c->p_qcw);
+  if (!st) st = alloc_n(c, c->pair_bufs, 2 * c->mcap, &c->p_qmask);
+  if (!st) st = alloc_n(c, c->pair_bufs, need_v, &c->p_val);
+  if (!st) st = alloc_n(c, c->pair_bufs, 2 * (uint64_t)c->ucap, &c->p_units);
+  if (!st) st = alloc_n(c, c->pair_bufs, 2 * (uint64_t)c->qcap, &c->p_q0);
+  if (!st) st = alloc_n(c, c->pair_bufs, 2 * (uint64_t)c->qcap, &c->p_q1);
+  c->pair_bytes = c->allocated - before;
+  if (st) {
     free_pair(c);
     return st;
   }

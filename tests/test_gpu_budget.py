@@ -67,3 +67,20 @@ def test_refused_batch_keeps_no_bytes(svv):
     ctx.set_tuning("batch_mode", 2)  # what needs no teams still runs
     np.testing.assert_array_equal(svv.to_u32(ctx.query(0, 0, 0, 8)), oracle.query(log, 0, 0, 0, 8))
     ctx.close()
+
+
+def test_regrown_pair_rows_are_counted_once(svv):
+    """A pair of longer windows replaces the pair arrays: the bytes held are
+    those of a context that ran the longer pair only."""
+    log = W.scaled_rmat(scale=12, edge_factor=8, n_snapshots=100, rate=0.002, seed=58, add_mode="skewed")
+    held = []
+    for lengths in ((100,), (8, 30, 100)):
+        with svv.Context(0) as ctx:
+            ctx.set_tuning("batch_mode", 2)
+            ctx.load_log(log)
+            for L in lengths:
+                outs, status = ctx.query_batch([(0, 0, 0, L), (0, 1, 0, L)])
+                assert status == [0, 0]
+                np.testing.assert_array_equal(svv.to_u32(outs[0]), oracle.query(log, 0, 0, 0, L))
+            held.append(ctx.device_bytes())
+    assert held[0] == held[1]
