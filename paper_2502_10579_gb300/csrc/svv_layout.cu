@@ -398,7 +398,7 @@ svv_status build_rowd(svv_ctx* c, const uint32_t* nfp, uint4* rowd) {
 // the layout itself is allocated.  Two copies to the host give the sizes; one
 // launch per step for both halves, since a small graph's load is bound by the
 // chain of launches (16 vertices, 64 edges: svv_load 0.57 -> 0.33 ms; 4,096 and
-// 32,768: 0.84 -> 0.60; one allocation for many arrays is a third of that).
+// 32,768: 0.84 -> 0.60, few allocations included).
 svv_status build_pull(svv_ctx* c) {
   const DevGraph& g = c->g;
   const uint32_t V = g.V;
